@@ -424,13 +424,18 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
     // Before the dependency wait this kernel reads only the segment tables
     // and the factors: the host launches it as a programmatic dependent only
     // when the previous kernel on the stream did not write those tables.
-    // The next kernel may be scheduled as soon as every CTA of this one runs.
-    pdl_launch_dependents();
+    // The next kernel may be scheduled as soon as every CTA of this one runs;
+    // after a shrink-only launch (whose dependent reads x before its own
+    // dependency wait) only once everything before this launch is complete.
+    if (!p.shrink_only) pdl_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n_blk = min(p.counts[3], p.w.blk_cap);
     if (p.counts[3] > p.w.blk_cap && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(p.err, SALT_DEVERR_RANK);
     const int nu = p.n_unit_prefix[p.n_proj];
-    if (n_blk <= 0 || nu <= 0) return;  // the same for every CTA
+    if (n_blk <= 0 || nu <= 0) {  // the same for every CTA
+        pdl_wait();  // a dependent of this launch relies on everything before it
+        return;
+    }
     const int n_bp = n_blk * p.n_proj;
     int KS = max(1, min(KS_MAX, (int)gridDim.x / n_bp));
     if (KS > 1 && (int64_t)n_bp * KS > p.w.part_cap) KS = max(1, p.w.part_cap / n_bp);
@@ -491,6 +496,7 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
     // barriers publish it; the x loads need not wait for it.)
     auto dep_wait = [&]() {
         pdl_wait();
+        if (p.shrink_only) pdl_launch_dependents();
         waited = true;
         if (tid == 0) info.epoch = *reinterpret_cast<volatile uint32_t *>(p.w.seq);
     };
@@ -1056,7 +1062,8 @@ cudaError_t apply_static_workspace(ApplyWork *out)
     return cudaSuccess;
 }
 
-cudaError_t encode_base_map(CUtensorMap *out, const uint16_t *W, int d_in, int d_out, int layout)
+cudaError_t encode_map_2d(CUtensorMap *out, const uint16_t *base, int64_t cols, int64_t rows, uint32_t box_cols,
+                          uint32_t box_rows)
 {
     using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
@@ -1073,14 +1080,11 @@ cudaError_t encode_base_map(CUtensorMap *out, const uint16_t *W, int d_in, int d
             encode = reinterpret_cast<Encode>(fn);
         }
     }
-    // IN_OUT: [d_in][d_out], inner dimension N, box 64 N x 64 K;
-    // OUT_IN: [d_out][d_in], inner dimension K, box 64 K x 128 N
-    const bool in_out = layout == SALT_W_IN_OUT;
-    const cuuint64_t dims[2] = {(cuuint64_t)(in_out ? d_out : d_in), (cuuint64_t)(in_out ? d_in : d_out)};
-    const cuuint64_t strides[1] = {(cuuint64_t)(in_out ? d_out : d_in) * 2};
-    const cuuint32_t box[2] = {64, in_out ? 64u : 128u};
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
+    const cuuint32_t box[2] = {box_cols, box_rows};
     const cuuint32_t es[2] = {1, 1};
-    const CUresult r = encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t *>(W), dims, strides, box, es,
+    const CUresult r = encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t *>(base), dims, strides, box, es,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
@@ -1088,30 +1092,8 @@ cudaError_t encode_base_map(CUtensorMap *out, const uint16_t *W, int d_in, int d
 
 cudaError_t apply_encode_vmap(ApplyWork &w)
 {
-    using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static Encode encode = nullptr;
-    static std::mutex mu;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (!encode) {
-            void *fn = nullptr;
-            cudaDriverEntryPointQueryResult q;
-            cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q);
-            if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return e != cudaSuccess ? e : cudaErrorNotSupported;
-            encode = reinterpret_cast<Encode>(fn);
-        }
-    }
     if (w.max_group < 1 || w.max_group > SALT_MAX_GROUP || w.blk_cap < 1) return cudaErrorInvalidValue;
-    const cuuint64_t dims[2] = {(cuuint64_t)VEXT_COLS, (cuuint64_t)w.max_group * w.blk_cap * TM};
-    const cuuint64_t strides[1] = {(cuuint64_t)VEXT_COLS * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)TM};
-    const cuuint32_t es[2] = {1, 1};
-    const CUresult r = encode(&w.vmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w.vext, dims, strides, box, es,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+    return encode_map_2d(&w.vmap, w.vext, VEXT_COLS, (int64_t)w.max_group * w.blk_cap * TM, 64, (uint32_t)TM);
 }
 
 cudaError_t apply_prepare(int device)

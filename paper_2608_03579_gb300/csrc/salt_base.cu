@@ -7,23 +7,38 @@
 // y is written, never read.  The low-rank part reuses the apply path's row
 // blocks: a shrink-only launch of the apply kernel leaves every block's V_ext
 // tile (scaled and masked as in the apply) in the segments workspace; this
-// kernel then runs the GEMM over 128-token tiles in grouped order and, for
-// every row block overlapping a tile, adds V_ext * Stack_B into the same
-// tensor-memory accumulator: one more group of MMAs whose A operand holds the
-// block's V rows at their tile rows and zeros elsewhere.  Tokens with no
-// term are in no block and get x W_base alone.
+// kernel runs the GEMM over tiles of tokens in grouped order and, for every
+// row block overlapping a tile, adds V_ext * Stack_B into the same
+// tensor-memory accumulator: further K chunks whose A operand holds the
+// block's V rows at their tile rows and zeros elsewhere.  Tokens with no term
+// are in no block and get x W_base alone.
 //
-// One persistent CTA per SM over the (M tile, N tile) pairs, 12 warps in
-// fixed roles:
-//   producers (warps 0-6): per 64-wide K chunk, the tile's x rows (gathered
-//       through the grouped order, cp.async) and the W tile (TMA: either
-//       layout lands in the layout its UMMA descriptor reads); then per
-//       overlapping block its V rows and stacked B columns (cp.async);
-//   MMA (warp 7): tcgen05.mma into one of two 128-column accumulators;
-//   epilogue (warps 8-11): one token row a thread, fp32 -> bf16 (RNE), store.
+// CG = 2 (batches of more than 128 tokens): a cluster of two CTAs computes a
+// 256-token x BN tile with cta_group::2 MMAs.  Each CTA loads its own 128
+// token rows and half of the W columns, so a 64-wide K chunk moves 32 KB into
+// each SM per 512 tensor cycles at BN = 256 (a 128 x 128 tile of one CTA
+// moves the same per 256, which bound the GEMM on L2-to-SM traffic).
+// CG = 1 (up to 128 tokens): one CTA, 128 x BN; only the batch's rows are
+// loaded, the tile is bound by streaming W.
+//
+// Persistent CTAs over units (tile, K split of KS).  Warp roles:
+//   warp 0      TMA of the W tile (either layout lands as its UMMA descriptor
+//               reads it);
+//   warp 1      tcgen05.mma into one of two BN-column accumulators;
+//   warps 2-7   everything gathered, by cp.async, a whole stage a warp (six
+//               stages in flight): the token rows of a K chunk, or a delta
+//               chunk's V rows and stacked B rows;
+//   warps 8-11  epilogue: fp32 -> bf16 (RNE) and store, one token row a
+//               thread; with K splits the fp32 partial goes to the workspace
+//               and the split that finishes last sums the tile's partials in
+//               split order (so the result does not depend on timing).
+// The launch is a programmatic dependent of the shrink, which releases it
+// once everything before the shrink is complete: the K loop over x and W
+// overlaps the shrink's tail, and only the delta and the partial stores wait
+// for the shrink itself.
 #include <cuda_bf16.h>
 
-#include <mutex>
+#include <algorithm>
 
 #include "salt_async.cuh"
 #include "salt_internal.cuh"
@@ -33,32 +48,33 @@
 namespace salt {
 namespace {
 
-constexpr int BM = 128;                    // tokens per tile (the UMMA M)
-constexpr int BN = 128;                    // output columns per tile
+constexpr int BM = 128;                    // token rows per CTA (the UMMA M is BM * CG)
 constexpr int BK = 64;                     // K chunk (128-byte rows)
-constexpr int NST = 4;                     // K stages in flight
-constexpr int X_BYTES = BM * 128;          // x rows of a chunk
-constexpr int W_BYTES = BN * 128;          // W tile of a chunk (either layout)
-constexpr int STAGE = X_BYTES + W_BYTES;
-constexpr int DV_BYTES = 2 * BM * 128;     // delta A operand: V rows, K 0..63 and 64..127
-constexpr int DB_BYTES = 2 * S_MAX * 128;  // delta B operand: stacked B rows, N 0..63 and 64..127
+constexpr int NST_MAX = 10;
+constexpr int BASE_RING = 208 * 1024;      // shared-memory ring
 constexpr int BASE_THREADS = 384;
-constexpr int PW = 7;                      // producer warps
-constexpr int PT = 32 * PW;
-constexpr int MW = 7;                      // the MMA warp
+constexpr int GW0 = 2, GWN = 6;            // gather warps; the ring holds at least as many stages (below)
 constexpr int EW0 = 8;                     // first epilogue warp
-constexpr int BAR_P = 1;                   // named barrier of the producers
+constexpr int EPI_N = 128;
+constexpr int BAR_E = 1;                   // named barrier of the epilogue warps
+constexpr int MT_MAX = SALT_MAX_TOKENS / BM;
+constexpr int BASE_KS_MAX = 16;
 
 struct BaseInfo {
-    uint64_t full[NST], empty[NST];
-    uint64_t dfull, dempty;
+    uint64_t full[NST_MAX], empty[NST_MAX];
     uint64_t accf[2], acce[2];
-    const uint16_t *bsrc[S_MAX];  // stacked B rows of the current block
-    int32_t prow[BM];             // x rows of the current tile (-1: past the batch)
+    int32_t ksteps[NST_MAX];               // a delta stage's K = 16 steps
+    int32_t mt_b0[MT_MAX], mt_b1[MT_MAX];  // row blocks overlapping M tile: [b0, b1)
+    int32_t mt_nd[MT_MAX];                 // its delta chunks
     uint32_t tmem;
+    int32_t last;
 };
-constexpr size_t BASE_SMEM = 1024 + NST * STAGE + DV_BYTES + DB_BYTES + (sizeof(BaseInfo) + 127) / 128 * 128;
+constexpr size_t BASE_SMEM = 1024 + BASE_RING + (sizeof(BaseInfo) + 127) / 128 * 128;
 static_assert(BASE_SMEM <= 227 * 1024, "shared memory exceeds the per-block limit");
+// A gather warp fills every GWN-th stage and waits only for its own slots'
+// phases; with at least GWN stages a slot's barrier is never two phases
+// behind the one it waits for (a parity wait could not tell).
+static_assert(BASE_RING / (2 * BM * 128) >= GWN, "stages for the gather warps");
 
 __device__ __forceinline__ const uint16_t *res_b_row(const BaseParams &p, int e)
 {
@@ -68,224 +84,476 @@ __device__ __forceinline__ const uint16_t *res_b_row(const BaseParams &p, int e)
     return base + (int64_t)rank * p.d_in + (int64_t)k * p.d_out;
 }
 
-// Row blocks overlapping grouped positions [m0, m0 + BM): [*b0, *b1).
-__device__ __forceinline__ void blocks_of_tile(const BaseParams &p, int n_blk, int m0, int &b0, int &b1)
+// 32 consecutive bytes of an output row
+__device__ __forceinline__ void store32(uint16_t *dst, const uint32_t (&w)[8], bool wide)
 {
-    // first block ending after m0 (blocks lie in grouped order)
-    int lo = 0, hi = n_blk;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        const int end = p.blk[BLK_INTS * mid + BLK_START] + p.blk[BLK_INTS * mid + BLK_LEN];
-        if (end <= m0) lo = mid + 1; else hi = mid;
+    if (wide) {
+        asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                     "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
+    } else {
+        *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4 *>(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
     }
-    b0 = lo;
-    b1 = lo;
-    while (b1 < n_blk && p.blk[BLK_INTS * b1 + BLK_START] < m0 + BM) ++b1;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b)
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+// A position in the ring of n stages and its phase parity.
+struct RingPos {
+    uint32_t slot = 0, phase = 0;
+    __device__ __forceinline__ void advance(uint32_t by, uint32_t n)
+    {
+        for (slot += by; slot >= n; slot -= n) phase ^= 1u;
+    }
+};
+
+template <int CG>
 __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid_constant__ BaseParams p)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
     uint8_t *ring = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-    uint8_t *dv = ring + NST * STAGE;
-    uint8_t *db = dv + DV_BYTES;
-    BaseInfo &info = *reinterpret_cast<BaseInfo *>(db + DB_BYTES);
-    const uint32_t ring32 = smem_u32(ring), dv32 = smem_u32(dv), db32 = smem_u32(db);
+    BaseInfo &info = *reinterpret_cast<BaseInfo *>(ring + BASE_RING);
+    const uint32_t ring32 = smem_u32(ring);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int T = p.T, n_blk = min(p.counts[3], p.blk_cap);
-    const int n_mt = (T + BM - 1) / BM, n_nt = (p.d_out + BN - 1) / BN;
-    const int n_tiles = n_mt * n_nt;
+    const int rank = CG == 2 ? (int)cluster_ctarank() : 0;  // this CTA's half of the tile
+    const int cl = blockIdx.x / CG, n_cl = gridDim.x / CG;
+    const int T = p.T, BN = p.bn, NB = BN / CG;             // NB: W columns this CTA loads
+    const int n_mt = (T + BM * CG - 1) / (BM * CG), n_nt = (p.d_out + BN - 1) / BN;
+    const int KS = p.ks, n_units = n_mt * n_nt * KS;
     const int nk = (p.d_in + BK - 1) / BK;
-    if (T <= 0) return;
+    // a stage: the CTA's token rows (only as many as the batch can fill),
+    // then its W columns.  The UMMA reads 128 rows: with fewer loaded the
+    // rest are whatever follows, and reach only accumulator rows past T.
+    const int m_rows = CG == 2 ? BM : (min(T, BM) + 15) & ~15;
+    const uint32_t x_bytes = (uint32_t)m_rows * 128u, stage = x_bytes + (uint32_t)NB * 128u;
+    const uint32_t nst = min((uint32_t)NST_MAX, (uint32_t)BASE_RING / stage);
     auto bar = [](const uint64_t &b) { return smem_u32(&b); };
-    if (warp == MW) {
-        tmem_alloc(smem_u32(&info.tmem), 256);
-        tmem_relinquish();
+
+    pdl_launch_dependents();
+    if (warp == 1) {
+        tmem_alloc<CG>(smem_u32(&info.tmem), 2 * BN);
+        tmem_relinquish<CG>();
     }
     if (tid == 0) {
-        for (int i = 0; i < NST; ++i) {
-            mbar_init(bar(info.full[i]), PT + 1);  // every producer's copies + the W tile's bytes
+        for (int i = 0; i < NST_MAX; ++i) {
+            mbar_init(bar(info.full[i]), 2 * CG);  // per CTA: the TMA warp and a gather warp
             mbar_init(bar(info.empty[i]), 1);
         }
-        mbar_init(bar(info.dfull), PT);
-        mbar_init(bar(info.dempty), 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(info.accf[i]), 1);
-            mbar_init(bar(info.acce[i]), 4);
+            mbar_init(bar(info.acce[i]), 4 * CG);
         }
         mbar_fence_init();
     }
-    tc_fence_before();
+    for (int i = tid; i < n_mt; i += BASE_THREADS) {
+        info.mt_b0[i] = 0x7fffffff;
+        info.mt_b1[i] = 0;
+        info.mt_nd[i] = 0;
+    }
     __syncthreads();
+    // Row blocks lie in grouped order and hold at most TM tokens, so each
+    // overlaps one or two M tiles.  (The segment tables are complete: they
+    // were written before the shrink started.)
+    const int n_blk = min(p.counts[3], p.blk_cap);
+    for (int b = tid; b < n_blk; b += BASE_THREADS) {
+        const int4 r = *reinterpret_cast<const int4 *>(p.blk + BLK_INTS * b);
+        const int S = r.w + p.blk[BLK_INTS * b + BLK_NRES];
+        if (S <= 0 || S > S_MAX || r.y <= 0) continue;  // flagged by the shrink
+        const int t0 = r.x / (BM * CG), t1 = (r.x + r.y - 1) / (BM * CG);
+        for (int t = t0; t <= t1; ++t) {
+            atomicMin(&info.mt_b0[t], b);
+            atomicMax(&info.mt_b1[t], b + 1);
+            atomicAdd(&info.mt_nd[t], (S + BK - 1) / BK);
+        }
+    }
+    tc_fence_before();
+    cta_or_cluster_sync<CG>();
     tc_fence_after();
     const uint32_t tmem = info.tmem;
-    bool ok_all = true;
+    bool ok = true;  // a bounded wait gave up: no further waits, no further loads
     auto wait_bar = [&](const uint64_t &b, uint32_t parity) {
-        if (!mbar_wait(smem_u32(&b), parity)) ok_all = false;
+        if (ok && !mbar_wait(smem_u32(&b), parity)) ok = false;
     };
-    // tile t: M tile t % n_mt, N tile t / n_mt (the M tiles of one W column
-    // block run side by side, so W is read from memory about once)
-    if (warp < PW) {
-        // ============================================================ producers
-        uint32_t g = 0, dg = 0;  // K stages and delta stages issued
-        for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-            const int m0 = (t % n_mt) * BM, n0 = (t / n_mt) * BN;
-            named_sync(BAR_P, PT);  // the previous tile's copies are out: the row table is free
-            if (tid < BM) info.prow[tid] = m0 + tid < T ? p.perm[m0 + tid] : -1;
-            named_sync(BAR_P, PT);
-            for (int kc = 0; kc < nk; ++kc, ++g) {
-                const uint32_t slot = g % NST;
-                if (g >= NST) wait_bar(info.empty[slot], ((g / NST) - 1) & 1);
-                const uint32_t xs = ring32 + slot * STAGE, ws = xs + X_BYTES;
-                const int k0 = kc * BK;
-                if (tid == 0) {
-                    mbar_expect_tx(bar(info.full[slot]), W_BYTES);
-                    if (p.w_layout == SALT_W_IN_OUT) {
-                        // W[d_in][d_out]: two boxes of 64 K rows x 64 N columns (MN-major)
-                        tma_load_2d(ws, &p.wmap, n0, k0, bar(info.full[slot]));
-                        tma_load_2d(ws + 64 * 128, &p.wmap, n0 + 64, k0, bar(info.full[slot]));
+    // unit u: tile u / KS (M tile tile % n_mt: the M tiles of one W column
+    // block run side by side, so W is read from memory about once), split u % KS
+    auto chunk_lo = [&](int s) { return nk * s / KS; };
+    const bool in_out = p.w_layout == SALT_W_IN_OUT;
+    auto n_delta = [&](int mt, int s) { const int nd = info.mt_nd[mt]; return nd > s ? (nd - s + KS - 1) / KS : 0; };
+
+    if (warp == 0) {
+        // ============================================================ TMA
+        RingPos rp;
+        bool wrapped = false;  // the ring's first round needs no wait
+        auto next_slot = [&]() {
+            if (wrapped) wait_bar(info.empty[rp.slot], rp.phase ^ 1u);
+        };
+        auto advance = [&]() {
+            rp.advance(1, nst);
+            wrapped = wrapped || rp.slot == 0;
+        };
+        if (lane == 0) {
+            for (int u = cl; u < n_units && ok; u += n_cl) {
+                const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
+                const int k1 = chunk_lo(s + 1);
+                for (int kc = chunk_lo(s); kc < k1 && ok; ++kc, advance()) {
+                    next_slot();
+                    if (!ok) break;
+                    const uint32_t ws = ring32 + rp.slot * stage + x_bytes;
+                    const uint32_t fb = leader_addr<CG>(bar(info.full[rp.slot]));
+                    const int k0 = kc * BK;
+                    mbar_expect_tx_cluster<CG>(fb, (uint32_t)NB * 128u);
+                    if (in_out) {
+                        // W[d_in][d_out]: boxes of 64 K rows x 64 N columns (MN-major)
+                        for (int h = 0; h < NB / 64; ++h) tma_load_2d_cg<CG>(ws + h * 8192, &p.wmap, n0 + 64 * h, k0, fb);
                     } else {
-                        // W[d_out][d_in]: one box of 128 N rows x 64 K (K-major)
-                        tma_load_2d(ws, &p.wmap, k0, n0, bar(info.full[slot]));
+                        // W[d_out][d_in]: one box of NB rows x 64 K (K-major)
+                        tma_load_2d_cg<CG>(ws, &p.wmap, k0, n0, fb);
                     }
                 }
-                for (int idx = tid; idx < BM * 8; idx += PT) {
-                    const int r = idx >> 3, c = idx & 7;
-                    const int row = info.prow[r];
-                    const bool ok = row >= 0 && k0 + c * 8 < p.d_in;
-                    cp_async16(xs + swz128(r, c), p.x + (ok ? (int64_t)row * p.d_in + k0 + c * 8 : 0), ok);
+                // the delta's stages hold nothing of W
+                for (int j = n_delta(mt, s); j > 0 && ok; --j, advance()) {
+                    next_slot();
+                    if (ok) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
                 }
-                cp_async_arrive_noinc(bar(info.full[slot]));
             }
-            // the delta of every row block overlapping the tile
-            int b0, b1;
-            blocks_of_tile(p, n_blk, m0, b0, b1);
-            for (int b = b0; b < b1; ++b) {
-                const int4 m0r = *reinterpret_cast<const int4 *>(p.blk + BLK_INTS * b);
-                const int start = m0r.x, M = m0r.y, d = m0r.z, rc = m0r.w;
-                const int S = rc + p.blk[BLK_INTS * b + BLK_NRES];
-                const int S_pad = (S + 15) & ~15;
-                if (S <= 0 || S > S_MAX) continue;  // flagged by the shrink
-                // the delta area's previous block has been consumed by the MMAs
-                if (dg > 0) wait_bar(info.dempty, (dg - 1) & 1);
-                named_sync(BAR_P, PT);
-                if (tid < S)
-                    info.bsrc[tid] = tid < rc ? p.B + ((int64_t)d * p.rc_max + tid) * p.d_out
-                                              : res_b_row(p, p.blk_res[(int64_t)b * S_MAX + (tid - rc)]);
-                named_sync(BAR_P, PT);
-                // V rows of the block at their tile rows (other rows zero), K-major halves
-                const uint16_t *vt = p.vext + (int64_t)b * (TM * VEXT_COLS);
-                for (int idx = tid; idx < BM * 16; idx += PT) {
-                    const int r = idx >> 4, c = idx & 15;  // c: 16-byte piece of the row's 256 bytes
-                    const int gp = m0 + r, i = gp - start;
-                    const bool ok = i >= 0 && i < M && c * 8 < S_pad;
-                    cp_async16(dv32 + (c >> 3) * (BM * 128) + swz128(r, c & 7), vt + (ok ? i * VEXT_COLS + c * 8 : 0), ok);
-                }
-                // stacked B rows, columns n0 .. n0 + 127 as two MN-major halves
-                for (int idx = tid; idx < S_pad * 16; idx += PT) {
-                    const int k = idx >> 4, c = idx & 15, col = n0 + c * 8;
-                    const bool ok = k < S && col < p.d_out;
-                    cp_async16(db32 + (c >> 3) * (S_MAX * 128) + swz128(k, c & 7), ok ? info.bsrc[k] + col : p.x, ok);
-                }
-                cp_async_arrive_noinc(bar(info.dfull));
-                ++dg;
-            }
+            // every stage released (with CG = 2 by the pair's first CTA, whose
+            // arrivals must find this CTA's barriers alive)
+            for (uint32_t i = 0; i < nst; ++i, advance())
+                if (wrapped) wait_bar(info.empty[rp.slot], rp.phase ^ 1u);
         }
-        cp_async_wait<0>();
-    } else if (warp == MW) {
+        __syncwarp();
+    } else if (warp == 1) {
         // ============================================================ MMA issue
-        if (lane == 0) {
-            const uint32_t id_k = idesc_bf16_f32(BM, BN);          // W K-major (N = 128)
-            const uint32_t id_mn = idesc_bf16_f32_bmn(BM, 64);     // W / stacked B MN-major, N = 64 per half
-            uint32_t g = 0, dg = 0, lt = 0;
-            for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++lt) {
-                const int m0 = (t % n_mt) * BM;
+        if (lane == 0 && rank == 0) {
+            const uint32_t id_k = idesc_bf16_f32(BM * CG, BN), id_mn = idesc_bf16_f32_bmn(BM * CG, BN);
+            // descriptors of the ring's first stage; a stage adds stage / 16, a
+            // K step 2 (K-major: 32 bytes) or 128 (MN-major: 16 rows)
+            const uint64_t x0 = sdesc_kmajor_sw128(ring32), wk0 = sdesc_kmajor_sw128(ring32 + x_bytes);
+            const uint64_t wmn0 = sdesc_mnmajor_sw128_lbo(ring32 + x_bytes, 8192);
+            const uint32_t st16 = stage >> 4;
+            RingPos rp;
+            uint32_t lt = 0;
+            for (int u = cl; u < n_units; u += n_cl, ++lt) {
+                const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt;
                 const uint32_t buf = lt & 1, acc = tmem + buf * BN;
                 if (lt >= 2) wait_bar(info.acce[buf], ((lt - 2) >> 1) & 1);
                 tc_fence_after();
-                for (int kc = 0; kc < nk; ++kc, ++g) {
-                    const uint32_t slot = g % NST;
-                    wait_bar(info.full[slot], (g / NST) & 1);
-                    fence_async_smem();
+                uint32_t accum = 0;
+                for (int n = chunk_lo(s + 1) - chunk_lo(s); n > 0; --n, rp.advance(1, nst)) {
+                    wait_bar(info.full[rp.slot], rp.phase);
                     tc_fence_after();
-                    const uint32_t xs = ring32 + slot * STAGE, ws = xs + X_BYTES;
+                    const uint64_t xd = x0 + rp.slot * st16;
+                    if (in_out) {
+                        const uint64_t wd = wmn0 + rp.slot * st16;
 #pragma unroll
-                    for (int kk = 0; kk < BK / 16; ++kk) {
-                        const uint32_t a = (kc > 0 || kk > 0) ? 1u : 0u;
-                        const uint64_t ad = sdesc_kmajor_sw128(xs + kk * 32);
-                        if (p.w_layout == SALT_W_IN_OUT) {
-                            umma_bf16(acc, ad, sdesc_mnmajor_sw128(ws + kk * 2048), id_mn, a);
-                            umma_bf16(acc + 64, ad, sdesc_mnmajor_sw128(ws + 64 * 128 + kk * 2048), id_mn, a);
-                        } else {
-                            umma_bf16(acc, ad, sdesc_kmajor_sw128(ws + kk * 32), id_k, a);
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, accum);
+                            accum = 1;
+                        }
+                    } else {
+                        const uint64_t wd = wk0 + rp.slot * st16;
+#pragma unroll
+                        for (int kk = 0; kk < BK / 16; ++kk) {
+                            umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 2, id_k, accum);
+                            accum = 1;
                         }
                     }
-                    umma_commit(bar(info.empty[slot]));
+                    umma_commit_cg<CG>(bar(info.empty[rp.slot]));
                 }
-                int b0, b1;
-                blocks_of_tile(p, n_blk, m0, b0, b1);
-                for (int b = b0; b < b1; ++b) {
-                    const int rc = p.blk[BLK_INTS * b + BLK_RC];
-                    const int S = rc + p.blk[BLK_INTS * b + BLK_NRES];
-                    if (S <= 0 || S > S_MAX) continue;
-                    const int S_pad = (S + 15) & ~15;
-                    wait_bar(info.dfull, dg & 1);
-                    fence_async_smem();
+                for (int n = n_delta(mt, s); n > 0; --n, rp.advance(1, nst)) {
+                    wait_bar(info.full[rp.slot], rp.phase);
                     tc_fence_after();
-                    for (int ks = 0; ks < (S_pad >> 4); ++ks) {
-                        const uint64_t ad = sdesc_kmajor_sw128(dv32 + (ks >> 2) * (BM * 128) + (ks & 3) * 32);
-                        umma_bf16(acc, ad, sdesc_mnmajor_sw128(db32 + ks * 2048), id_mn, 1u);
-                        umma_bf16(acc + 64, ad, sdesc_mnmajor_sw128(db32 + S_MAX * 128 + ks * 2048), id_mn, 1u);
+                    const uint64_t xd = x0 + rp.slot * st16, wd = wmn0 + rp.slot * st16;
+                    const int steps = ok ? *reinterpret_cast<volatile int32_t *>(&info.ksteps[rp.slot]) : 0;
+                    for (int kk = 0; kk < steps; ++kk) {
+                        umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, accum);
+                        accum = 1;
                     }
-                    umma_commit(bar(info.dempty));
-                    ++dg;
+                    umma_commit_cg<CG>(bar(info.empty[rp.slot]));
                 }
-                umma_commit(bar(info.accf[buf]));
+                umma_commit_cg<CG>(bar(info.accf[buf]));
             }
         }
         __syncwarp();
+    } else if (warp < EW0) {
+        // ============================================================ gathers
+        // Stage g (counted over the CTA's units) belongs to warp g % GWN.
+        const int w = warp - GW0;
+        RingPos rp;                 // the warp's next stage
+        rp.advance(w, nst);
+        uint32_t mine = w;          // stages until the warp's next one
+        bool wrapped = false, v_ready = false;
+        auto begin = [&]() {        // the stage's slot is free
+            if (wrapped) wait_bar(info.empty[rp.slot], rp.phase ^ 1u);
+            ok = __all_sync(0xffffffffu, ok);
+        };
+        auto finish = [&]() {       // the warp's copies have landed; on to its next stage
+            cp_async_commit();
+            cp_async_wait<0>();
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
+            const uint32_t before = rp.slot;
+            rp.advance(GWN, nst);
+            wrapped = wrapped || rp.slot <= before;
+            mine += GWN;
+        };
+        uint32_t xoff[BM / 4];      // this lane's token rows (row 4 i + lane / 8), in 16-byte units of x
+        int mt_of = -1, rows = 0;
+        const uint32_t d16 = (uint32_t)p.d_in >> 3;
+        for (int u = cl; u < n_units && ok; u += n_cl) {
+            const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
+            const int m0 = (mt * CG + rank) * BM;
+            if (mt != mt_of) {
+                mt_of = mt;
+                rows = max(0, min(BM, T - m0));
+#pragma unroll
+                for (int i = 0; i < BM / 4; ++i) {
+                    const int r = 4 * i + (lane >> 3);
+                    xoff[i] = r < rows ? (uint32_t)p.perm[m0 + r] : 0u;
+                }
+#pragma unroll
+                for (int i = 0; i < BM / 4; ++i) xoff[i] = xoff[i] * d16 + (uint32_t)(lane & 7);
+            }
+            const int k0 = chunk_lo(s), n = chunk_lo(s + 1) - k0;
+            const uint32_t sw = (uint32_t)swz128(lane >> 3, lane & 7);  // row 4 i + lane / 8: swizzle by (4 i + lane / 8) % 8
+            while ((int)mine < n && ok) {
+                begin();
+                if (!ok) break;
+                const int kc = k0 + (int)mine;
+                const uint32_t xs = ring32 + rp.slot * stage;
+                const bool in = kc * BK + (lane & 7) * 8 < p.d_in;
+                const uint16_t *xk = p.x + (in ? (int64_t)kc * BK : 0);
+#pragma unroll
+                for (int i = 0; i < BM / 4; ++i)
+                    if (4 * i + (lane >> 3) < rows)
+                        cp_async16(xs + ((sw + i * 512) ^ ((i & 1) << 6)), xk + (uint64_t)xoff[i] * 8, in);
+                finish();
+            }
+            mine -= n;
+            // delta chunk j of the tile belongs to split j % KS
+            const int b1 = info.mt_b1[mt];
+            int j = 0;
+            if (n_delta(mt, s) > 0 && !v_ready) {
+                pdl_wait();  // the V tiles are the shrink's
+                v_ready = true;
+            }
+            for (int bb = info.mt_b0[mt]; bb < b1 && ok; bb += 32) {
+                // 32 blocks at a time: lane l holds block bb + l
+                int4 r0 = make_int4(0, 0, -1, 0);
+                int S = 0;
+                if (bb + lane < b1) {
+                    r0 = *reinterpret_cast<const int4 *>(p.blk + BLK_INTS * (bb + lane));
+                    S = r0.w + p.blk[BLK_INTS * (bb + lane) + BLK_NRES];
+                    if (S > S_MAX || S <= 0 || r0.y <= 0) S = 0;
+                }
+                const int nb = min(32, b1 - bb);
+                for (int i = 0; i < nb && ok; ++i) {
+                    const int Sb = __shfl_sync(0xffffffffu, S, i);
+                    for (int c0 = 0; c0 < Sb; c0 += BK, ++j) {
+                        if (j % KS != s) continue;
+                        if (mine > 0) {
+                            --mine;
+                            continue;
+                        }
+                        const int start = __shfl_sync(0xffffffffu, r0.x, i), M = __shfl_sync(0xffffffffu, r0.y, i);
+                        const int d = __shfl_sync(0xffffffffu, r0.z, i), rc = __shfl_sync(0xffffffffu, r0.w, i);
+                        const int b = bb + i, kn = min(BK, ((Sb + 15) & ~15) - c0);  // stack rows, padded to 16
+                        // the lane's two stacked B rows
+                        const uint16_t *src[2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int k = c0 + h * 32 + lane;
+                            src[h] = k >= Sb ? nullptr
+                                     : k < rc ? p.B + ((int64_t)d * p.rc_max + k) * p.d_out
+                                              : res_b_row(p, p.blk_res[(int64_t)b * S_MAX + (k - rc)]);
+                        }
+                        begin();
+                        if (!ok) break;
+                        const uint32_t xs = ring32 + rp.slot * stage, ws = xs + x_bytes;
+                        // V rows of the block at their tile rows (other rows zero)
+                        const uint16_t *vt = p.vext + (int64_t)b * (TM * VEXT_COLS) + c0;
+                        for (int idx = lane; idx < m_rows * 8; idx += 32) {
+                            const int r = idx >> 3, c = idx & 7, iv = m0 + r - start;
+                            const bool in = iv >= 0 && iv < M && c * 8 < kn;
+                            cp_async16(xs + swz128(r, c), vt + (in ? iv * VEXT_COLS + c * 8 : 0), in);
+                        }
+                        // stacked B rows, this CTA's columns, as 64-wide MN-major parts;
+                        // 8 or 16 pieces of 16 bytes a row (kn times that is a
+                        // multiple of 32: every lane takes part in every round)
+                        const int lg = NB == 128 ? 4 : 3;
+                        for (int idx = lane; idx < kn << lg; idx += 32) {
+                            const int k = idx >> lg, c = idx & ((1 << lg) - 1), col = n0 + c * 8;
+                            const uint64_t lo = (uint64_t)__shfl_sync(0xffffffffu, (unsigned long long)src[0], k & 31);
+                            const uint64_t hi = (uint64_t)__shfl_sync(0xffffffffu, (unsigned long long)src[1], k & 31);
+                            const uint16_t *sp = reinterpret_cast<const uint16_t *>(k < 32 ? lo : hi);
+                            const bool in = sp != nullptr && col < p.d_out;
+                            cp_async16(ws + (c >> 3) * 8192 + swz128(k, c & 7), in ? sp + col : p.x, in);
+                        }
+                        if (lane == 0) info.ksteps[rp.slot] = kn >> 4;
+                        finish();
+                        mine -= 1;  // this stage itself
+                    }
+                }
+            }
+        }
     } else {
         // ============================================================ epilogue
-        const int q = warp & 3, row = q * 32 + lane;
+        const int q = warp & 3, row = q * 32 + lane, et = tid - 32 * EW0;
+        const bool wide = (p.d_out & 15) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 31) == 0;
         uint32_t lt = 0;
-        for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++lt) {
-            const int m0 = (t % n_mt) * BM, n0 = (t / n_mt) * BN;
+        if (KS > 1) pdl_wait();  // the partials' workspace is the shrink's
+        for (int u = cl; u < n_units; u += n_cl, ++lt) {
+            const int tile = u / KS, mt = tile % n_mt, n0 = tile / n_mt * BN;
             const uint32_t buf = lt & 1;
-            const int gp = m0 + row;
+            const int m0 = (mt * CG + rank) * BM, gp = m0 + row;
             const int tok = gp < T ? p.perm[gp] : -1;
             wait_bar(info.accf[buf], (lt >> 1) & 1);
             tc_fence_after();
-            uint16_t *yr = tok >= 0 ? p.y + (int64_t)tok * p.d_out : nullptr;
+            const uint32_t ta = tmem + ((uint32_t)(q * 32) << 16) + buf * BN;
+            const int rows = max(0, min(BM, T - m0));
+            float *part = p.part + ((int64_t)u * CG + rank) * (m_rows * BN);
+            uint16_t *yr = p.y + (int64_t)max(tok, 0) * p.d_out;
+            if (q * 32 < rows) {
 #pragma unroll 1
-            for (int c16 = 0; c16 < BN / 16; ++c16) {
-                uint32_t v[16];
-                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + buf * BN + c16 * 16, v);
-                tmem_ld_wait();
-                const int col = n0 + c16 * 16;
-                if (yr) {
-                    uint32_t w[8];
+                for (int c = 0; c < BN; c += 32) {
+                    uint32_t v[2][16];
+                    tmem_ld16(ta + c, v[0]);
+                    tmem_ld16(ta + c + 16, v[1]);
+                    tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const __nv_bfloat162 h =
-                            __floats2bfloat162_rn(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-                        w[i] = *reinterpret_cast<const uint32_t *>(&h);
+                    for (int h = 0; h < 2; ++h) {
+                        const int col = n0 + c + 16 * h;
+                        if (tok < 0) continue;
+                        if (KS > 1) {
+                            float4 *dst = reinterpret_cast<float4 *>(part + row * BN + c + 16 * h);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                __stcg(dst + i, make_float4(__uint_as_float(v[h][4 * i]), __uint_as_float(v[h][4 * i + 1]),
+                                                            __uint_as_float(v[h][4 * i + 2]), __uint_as_float(v[h][4 * i + 3])));
+                            continue;
+                        }
+                        uint32_t w[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            w[i] = pack_bf16(__uint_as_float(v[h][2 * i]), __uint_as_float(v[h][2 * i + 1]));
+                        if (col + 8 < p.d_out) store32(yr + col, w, wide);
+                        else if (col < p.d_out) *reinterpret_cast<uint4 *>(yr + col) = make_uint4(w[0], w[1], w[2], w[3]);
                     }
-                    if (col < p.d_out) *reinterpret_cast<uint4 *>(yr + col) = make_uint4(w[0], w[1], w[2], w[3]);
-                    if (col + 8 < p.d_out) *reinterpret_cast<uint4 *>(yr + col + 8) = make_uint4(w[4], w[5], w[6], w[7]);
                 }
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_relaxed(bar(info.acce[buf]));
+            if (lane == 0) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.acce[buf])));
+            if (KS == 1) continue;
+            // the split that finishes the tile last (this CTA's rows) sums its partials
+            __threadfence();
+            named_sync(BAR_E, EPI_N);
+            if (et == 0) {
+                uint32_t *ctr = p.ctr + (tile * CG + rank);
+                const uint32_t n = atomicAdd(ctr, 1u);
+                info.last = n == (uint32_t)KS - 1u;
+                if (info.last) atomicExch(ctr, 0u);  // zero for the next launch
+                __threadfence();
+            }
+            named_sync(BAR_E, EPI_N);
+            if (!info.last) continue;
+            const float *p0 = p.part + ((int64_t)tile * KS * CG + rank) * (m_rows * BN);
+            const int64_t ps = (int64_t)CG * m_rows * BN;
+            const int cpr = BN >> 3, n_it = rows * cpr;
+            // (row, 8 columns) items, two a round per thread, up to four splits' loads in flight
+            for (int base = et; base < n_it; base += 2 * EPI_N) {
+                float a[2][8] = {};
+                for (int s0 = 0; s0 < KS; s0 += 4) {
+                    float4 v[2][4][2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) {
+                            const int it = base + h * EPI_N;
+                            if (it < n_it && s0 + s < KS) {
+                                const float4 *src = reinterpret_cast<const float4 *>(p0 + (s0 + s) * ps + (int64_t)it * 8);
+                                v[h][s][0] = __ldcg(src);
+                                v[h][s][1] = __ldcg(src + 1);
+                            } else {
+                                v[h][s][0] = v[h][s][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
+                        }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) {
+                            a[h][0] += v[h][s][0].x;
+                            a[h][1] += v[h][s][0].y;
+                            a[h][2] += v[h][s][0].z;
+                            a[h][3] += v[h][s][0].w;
+                            a[h][4] += v[h][s][1].x;
+                            a[h][5] += v[h][s][1].y;
+                            a[h][6] += v[h][s][1].z;
+                            a[h][7] += v[h][s][1].w;
+                        }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int it = base + h * EPI_N;
+                    if (it >= n_it) continue;
+                    const int r = it / cpr, col = n0 + (it - r * cpr) * 8;
+                    if (col < p.d_out)
+                        *reinterpret_cast<uint4 *>(p.y + (int64_t)p.perm[m0 + r] * p.d_out + col) =
+                            make_uint4(pack_bf16(a[h][0], a[h][1]), pack_bf16(a[h][2], a[h][3]),
+                                       pack_bf16(a[h][4], a[h][5]), pack_bf16(a[h][6], a[h][7]));
+                }
+            }
         }
     }
+    pdl_wait();  // the launch completes after the shrink has
+    if (!ok) {
+        atomicOr(p.err, SALT_DEVERR_TIMEOUT);
+        __nanosleep(1000000);  // copies already issued land before the CTA may exit
+    }
+    __syncwarp();
     tc_fence_before();
-    __syncthreads();
-    if (warp == MW) tmem_dealloc(tmem, 256);
-    if (!ok_all) atomicOr(p.err, SALT_DEVERR_TIMEOUT);
+    cta_or_cluster_sync<CG>();
+    if (warp == 1) tmem_dealloc<CG>(tmem, 2 * BN);
 }
 
 int g_base_sms[64];
+
+struct BasePlan {
+    int cg, bn, ks;
+};
+
+// The tile and the K splits of a launch, by an estimate of its tensor
+// cycles: whole waves of units over the SMs (pairs of SMs for CG = 2), a
+// chunk's cost, a fixed cost per wave and, with splits, the partials' way
+// through L2.
+BasePlan base_plan(int T, int d_in, int d_out, int n_sm, int part_floats)
+{
+    const int nk = (d_in + BK - 1) / BK, cg = T > BM ? 2 : 1, n_cl = std::max(1, n_sm / cg);
+    const int n_mt = (T + BM * cg - 1) / (BM * cg), m_rows = cg == 2 ? BM : (std::min(T, BM) + 15) & ~15;
+    BasePlan best = {cg, 128, 1};
+    double best_cost = 1e30;
+    for (int bn = 128; bn <= (cg == 2 ? 256 : 128); bn *= 2) {
+        const int n_nt = (d_out + bn - 1) / bn;
+        for (int ks = 1; ks <= std::min(BASE_KS_MAX, nk); ++ks) {
+            const int64_t tiles = (int64_t)n_mt * n_nt, units = tiles * ks;
+            if (ks > 1 && (units * cg * m_rows * bn > part_floats || tiles * cg > BASE_CTRS)) break;
+            const double waves = (double)((units + n_cl - 1) / n_cl);
+            const double chunk = cg == 2 ? (bn == 256 ? 560 : 340) : 600;
+            const double split = ks > 1 ? (double)m_rows * bn * (0.06 + 0.06 * ks) + 3000 : 0;
+            const double cost = waves * (((nk + ks - 1) / ks) * chunk + 500) + split;
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = {cg, bn, ks};
+            }
+        }
+    }
+    return best;
+}
 
 }  // namespace
 
@@ -294,20 +562,45 @@ cudaError_t base_prepare(int device)
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
     cudaError_t e = cudaDeviceGetAttribute(&g_base_sms[device], cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(salt_base_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BASE_SMEM);
+    e = cudaFuncSetAttribute(salt_base_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BASE_SMEM);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(salt_base_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BASE_SMEM);
 }
 
-cudaError_t launch_base(const BaseParams &p, cudaStream_t stream)
+cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const int n_sm = (dev >= 0 && dev < 64 && g_base_sms[dev] > 0) ? g_base_sms[dev] : 1;
-    const int n_tiles = ((p.T + BM - 1) / BM) * ((p.d_out + BN - 1) / BN);
-    const int grid = n_tiles < n_sm ? n_tiles : n_sm;
-    if (grid <= 0) return cudaSuccess;
-    salt_base_kernel<<<grid, BASE_THREADS, BASE_SMEM, stream>>>(p);
-    return cudaGetLastError();
+    BasePlan pl = base_plan(p.T, p.d_in, p.d_out, n_sm, PART_CAP * TM * PART_COLS);
+    p.bn = pl.bn;
+    p.ks = pl.ks;
+    const cuuint32_t nb = (cuuint32_t)(pl.bn / pl.cg);
+    // W_base[d_in][d_out]: boxes of 64 K rows x 64 N columns;
+    // W_base[d_out][d_in]: NB rows x 64 K
+    e = p.w_layout == SALT_W_IN_OUT ? encode_map_2d(&p.wmap, W, p.d_out, p.d_in, 64, 64)
+                                    : encode_map_2d(&p.wmap, W, p.d_in, p.d_out, 64, nb);
+    if (e != cudaSuccess) return e;
+    const int bm = BM * pl.cg;
+    const int64_t units = (int64_t)((p.T + bm - 1) / bm) * ((p.d_out + pl.bn - 1) / pl.bn) * pl.ks;
+    const int n_cl = (int)std::min<int64_t>(units, std::max(1, n_sm / pl.cg));
+    if (n_cl <= 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = pl.cg;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(n_cl * pl.cg, 1, 1);
+    cfg.blockDim = dim3(BASE_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = BASE_SMEM;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return pl.cg == 2 ? cudaLaunchKernelEx(&cfg, salt_base_kernel<2>, p) : cudaLaunchKernelEx(&cfg, salt_base_kernel<1>, p);
 }
 
 }  // namespace salt

@@ -90,7 +90,8 @@ static_assert(SALT_MAX_RESIDUAL_RANK <= 128, "a residual row code holds ranks up
 //           a launch uses the half of its epoch's parity and zeroes the
 //           other half for the next launch;
 //   seq:    [0] launch counter (the epoch), [1] CTAs of the running launch
-//           that have finished.
+//           that have finished;
+//   base_ctr: the base-weight kernel's split counters (zero between launches).
 struct ApplyWork {
     // TMA map of vext as a 2-D bf16 tensor [rows][VEXT_COLS], box 64 x TM,
     // 128-byte swizzle (the K-major UMMA layout of a V tile half)
@@ -103,6 +104,7 @@ struct ApplyWork {
     uint32_t *arrive;      // [2 * SALT_MAX_GROUP * blk_cap]
     uint32_t *vdone;       // [2 * SALT_MAX_GROUP * blk_cap]
     uint32_t *seq;         // [2]
+    uint32_t *base_ctr;    // [BASE_CTRS] the base-weight kernel's split counters
 };
 constexpr int PART_COLS = SALT_MAX_TOKEN_RANK;  // centroid | own residual, per token
 static_assert(PART_COLS % 4 == 0, "partial rows are read as float4");
@@ -162,9 +164,10 @@ struct ApplyParams {
 // One projection of the base-weight GEMM fused with the SALT delta
 // (salt_lora_apply_with_base).
 struct BaseParams {
-    // W_base as a 2-D bf16 TMA map, 128-byte swizzle: for SALT_W_IN_OUT the
-    // tensor [d_in][d_out] with box 64 (N) x 64 (K); for SALT_W_OUT_IN the
-    // tensor [d_out][d_in] with box 64 (K) x 128 (N)
+    // W_base as a 2-D bf16 TMA map, 128-byte swizzle (encoded by
+    // launch_base): for SALT_W_IN_OUT the tensor [d_in][d_out] with box
+    // 64 (N) x 64 (K), for SALT_W_OUT_IN the tensor [d_out][d_in] with box
+    // 64 (K) x the W columns a CTA loads
     alignas(64) CUtensorMap wmap;
     const uint16_t *x;       // [T][d_in]
     uint16_t *y;             // [T][d_out], written
@@ -177,13 +180,20 @@ struct BaseParams {
     const uint8_t *pool;
     int64_t slot_stride;
     int64_t res_off;         // sum over earlier layers of (d_in + d_out), in elements
+    float *part;             // fp32 partials of the K splits (the apply's partial tiles)
+    uint32_t *ctr;           // [BASE_CTRS] splits finished, per (tile, CTA of the pair); zero between launches
     int32_t T, d_in, d_out, rc_max, w_layout, blk_cap;
+    int32_t bn, ks;          // tile columns and K splits (launch_base)
     uint32_t *err;
 };
+constexpr int BASE_CTRS = 1024;
 cudaError_t base_prepare(int device);
-cudaError_t launch_base(const BaseParams &p, cudaStream_t stream);
-// The base weight as the TMA map the fused kernel reads (host).
-cudaError_t encode_base_map(CUtensorMap *out, const uint16_t *W, int d_in, int d_out, int layout);
+// The GEMM over W, as a programmatic dependent of the shrink-only apply
+// launched just before it on the stream.
+cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream);
+// A row-major bf16 tensor [rows][cols] as a 2-D TMA map, 128-byte swizzle (host).
+cudaError_t encode_map_2d(CUtensorMap *out, const uint16_t *base, int64_t cols, int64_t rows, uint32_t box_cols,
+                          uint32_t box_rows);
 
 // Encode w.vmap over the max_group * blk_cap V tiles of w.vext (host; once
 // per workspace).

@@ -41,6 +41,20 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         "l"(map), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
+// The same into this CTA's shared memory; with CG = 2 the barrier may be the
+// peer's (a cluster address).
+template <int CG>
+__device__ __forceinline__ void tma_load_2d_cg(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar)
+{
+    if (CG == 1)
+        tma_load_2d(dst, map, x, y, bar);
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+            "%3}], [%4];\n" ::"r"(dst),
+            "l"(map), "r"(x), "r"(y), "r"(bar)
+            : "memory");
+}
 // barrier among the first n threads of the CTA (n a multiple of 32), id 1..15
 __device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(n) : "memory"); }
 // named barrier that also ANDs a predicate over its n threads: every thread

@@ -903,6 +903,8 @@ salt_status salt_segments_create(salt_ctx *ctx, salt_segments **out)
          cudaMemset(seg->work.arrive, 0, 2 * n_pairs * sizeof(uint32_t)) == cudaSuccess &&
          cudaMemset(seg->work.vdone, 0, 2 * n_pairs * sizeof(uint32_t)) == cudaSuccess &&
          cudaMemset(seg->work.seq, 0, 2 * sizeof(uint32_t)) == cudaSuccess &&
+         cudaMalloc(&seg->work.base_ctr, BASE_CTRS * sizeof(uint32_t)) == cudaSuccess &&
+         cudaMemset(seg->work.base_ctr, 0, BASE_CTRS * sizeof(uint32_t)) == cudaSuccess &&
          apply_encode_vmap(seg->work) == cudaSuccess;
     for (int i = 0; ok && i < 2; ++i) {
         ok = cudaHostAlloc(&seg->staging[i], 3 * (size_t)n * sizeof(int32_t), cudaHostAllocDefault) == cudaSuccess &&
@@ -943,6 +945,7 @@ void salt_segments_destroy(salt_segments *seg)
     cudaFree(seg->work.arrive);
     cudaFree(seg->work.vdone);
     cudaFree(seg->work.seq);
+    cudaFree(seg->work.base_ctr);
     for (int i = 0; i < 2; ++i) {
         if (seg->staging[i]) cudaFreeHost(seg->staging[i]);
         if (seg->staging_ev[i]) cudaEventDestroy(seg->staging_ev[i]);
@@ -1222,7 +1225,6 @@ salt_status salt_lora_apply_with_base(salt_ctx *ctx, const salt_segments *seg_, 
     BaseParams bp;
     std::memset(&bp, 0, sizeof bp);
     const int din = ctx->d_in[layer], dout = ctx->d_out[layer];
-    CUDA_OR_FAIL(ctx, encode_base_map(&bp.wmap, static_cast<const uint16_t *>(W), din, dout, layout));
     bp.x = static_cast<const uint16_t *>(x);
     bp.y = static_cast<uint16_t *>(y);
     bp.perm = seg->d.aperm;
@@ -1240,8 +1242,10 @@ salt_status salt_lora_apply_with_base(salt_ctx *ctx, const salt_segments *seg_, 
     bp.rc_max = ctx->rc_max;
     bp.w_layout = layout;
     bp.blk_cap = seg->work.blk_cap;
+    bp.part = seg->work.part;
+    bp.ctr = seg->work.base_ctr;
     bp.err = ctx->err_dev;
-    CUDA_OR_FAIL(ctx, launch_base(bp, static_cast<cudaStream_t>(stream_)));
+    CUDA_OR_FAIL(ctx, launch_base(bp, static_cast<const uint16_t *>(W), static_cast<cudaStream_t>(stream_)));
     return SALT_OK;
 }
 

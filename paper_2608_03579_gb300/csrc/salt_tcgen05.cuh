@@ -113,6 +113,14 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
 // The same with B MN-major (bit 16: B transposed).
 __host__ __device__ constexpr uint32_t idesc_bf16_f32_bmn(int M, int N) { return idesc_bf16_f32(M, N) | (1u << 16); }
 
+// MN-major operand whose MN extent spans several 64-wide atoms: lbo bytes
+// from one atom to the next, 1024 bytes between 8-deep K groups.
+__device__ __forceinline__ uint64_t sdesc_mnmajor_sw128_lbo(uint32_t saddr, uint32_t lbo)
+{
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
 // D[tmem] (+)= A * B^T for one K=16 step, issued by a single thread.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate)
@@ -127,6 +135,107 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
                  : "memory");
+}
+
+// ---------------------------------------------------------------- CTA pairs
+// The same operations for one CTA (CG = 1) or a cluster of two (CG = 2: a
+// pair shares an M = 256 MMA, each CTA holding 128 rows of A and D and half
+// of B's N; every tcgen05 operation of a kernel uses one cta_group).
+__device__ __forceinline__ uint32_t cluster_ctarank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(r));
+    return r;
+}
+// the cluster address of a barrier of the pair's first CTA (CG = 1: the CTA's own)
+template <int CG>
+__device__ __forceinline__ uint32_t leader_addr(uint32_t saddr)
+{
+    if (CG == 1) return saddr;
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(r) : "r"(saddr));
+    return r;
+}
+template <int CG>
+__device__ __forceinline__ void cta_or_cluster_sync()
+{
+    if (CG == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    }
+}
+// Arrivals on a barrier of either CTA of the pair (an address of
+// leader_addr).  A cluster-scope release in the thread that feeds every
+// stage was measured at 0.4 us a stage, so the TMA thread arrives relaxed:
+// what its stages guard is ordered by the copies' own completion.
+template <int CG>
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
+{
+    if (CG == 1) asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+    else asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+template <int CG>
+__device__ __forceinline__ void mbar_arrive_relaxed_cluster(uint32_t bar)
+{
+    if (CG == 1) asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+    else asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+template <int CG>
+__device__ __forceinline__ void mbar_expect_tx_cluster(uint32_t bar, uint32_t bytes)
+{
+    if (CG == 1)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+    else
+        asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
+                     : "memory");
+}
+// tensor-memory allocation: one warp of each CTA of the pair
+template <int CG>
+__device__ __forceinline__ void tmem_alloc(uint32_t dst, uint32_t ncols)
+{
+    if (CG == 1) asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dst), "r"(ncols));
+    else asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(dst), "r"(ncols));
+}
+template <int CG>
+__device__ __forceinline__ void tmem_relinquish()
+{
+    if (CG == 1) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::);
+    else asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::);
+}
+template <int CG>
+__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
+{
+    if (CG == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(ncols));
+    else asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(ncols));
+}
+template <int CG>
+__device__ __forceinline__ void umma_bf16_cg(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate)
+{
+    if (CG == 1) {
+        umma_bf16(d_tmem, adesc, bdesc, idesc, accumulate);
+    } else {
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+                d_tmem),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+    }
+}
+// arrive on the barrier at this address of every CTA of the pair once the
+// issuing thread's tcgen05 operations so far have completed
+template <int CG>
+__device__ __forceinline__ void umma_commit_cg(uint32_t bar)
+{
+    if (CG == 1) {
+        umma_commit(bar);
+    } else {
+        const uint16_t mask = 3;
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n" ::"r"(bar),
+            "h"(mask)
+            : "memory");
+    }
 }
 
 }  // namespace salt

@@ -98,3 +98,38 @@ def test_with_base_config3(salt_lib, oracle_mod, wl, layout):
             assert r.device_error() == 0
             assert_close(got[rows], _ref(oracle_mod, w, l, W, layout, rows=rows),
                          f"with base, config 3 {w.layers[l][0]}, layout {layout}")
+
+
+@pytest.mark.parametrize("T,d_in,d_out", [
+    (1, 64, 64),          # one token, one K chunk, half a tile of columns
+    (24, 4096, 256),      # few tiles: K splits, one CTA a tile
+    (127, 136, 136), (128, 1032, 392),    # the last batches of one CTA a tile; remainders in K and N
+    (129, 1032, 392),     # the first batch of CTA pairs: one token in the second half
+    (257, 72, 264), (300, 4096, 128),     # a second M tile with an empty second half; K splits of pairs
+    (700, 520, 1288),     # more stages than the ring, several units a pair
+])
+@pytest.mark.parametrize("layout", [0, 1])
+def test_with_base_tile_edges(salt_lib, oracle_mod, wl, layout, T, d_in, d_out):
+    """Every tile and split shape of the base kernel at its edges; users in
+    random order, stacks of one and of two 64-row chunks, tokens without a
+    term; run twice (the split counters must be left at zero)."""
+    from paper_2608_03579_gb300.runner import SaltRunner
+    n_users = 40
+    u = (wl.uniform(31, 1, T) * n_users).astype(np.int32) % n_users
+    dom, slot = (u % 2).astype(np.int32), u.copy()
+    none = wl.uniform(31, 2, T) < 0.1
+    dom[none], slot[none] = -1, -1
+    w = wl.Workload("base_edges", 31, [("p", d_in, d_out)], 2, [64, 5], n_users, [1, 2] * (n_users // 2),
+                    dom_ids=dom, slot_ids=slot)
+    w.y_mode = "zeros"
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        r.build()
+        W = _weight(wl, 31, d_in, d_out, layout)
+        got = _run(salt_lib, r, w, 0, W, layout)
+        again = _run(salt_lib, r, w, 0, W, layout)
+        assert r.device_error() == 0
+        assert salt_lib.salt_guard_check(r.ctx, r.seg) == 0
+    assert np.array_equal(got, again)
+    assert_close(got, _ref(oracle_mod, w, 0, W, layout), f"with base, {T} x {d_in} x {d_out}, layout {layout}")
