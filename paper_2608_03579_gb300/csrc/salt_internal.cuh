@@ -65,10 +65,12 @@ struct SegDev {
     // grouped order (perm); with them a user's tokens in several bins are
     // one run here, so they share one set of residual rows in a block.
     int32_t *aperm;        // [max_tokens] token index in apply order
-    int32_t *a_dptr;       // [max_tokens + 1] domain runs of the apply order (gamma builds)
-    int32_t *a_ddom;       // [max_tokens]
     int32_t *a_uptr;       // [max_tokens + 1] (domain, slot) runs of the apply order (gamma builds)
     int32_t *a_udom;       // [max_tokens]
+    // the apply order's user runs: the domain run each lies in, and a domain
+    // run's first user run
+    int32_t *u_drun;       // [max_tokens]
+    int32_t *d_first;      // [max_tokens]
 };
 
 // Code of one residual row of a factor stack: row k of the rank-`rank`

@@ -888,8 +888,8 @@ salt_status salt_segments_create(salt_ctx *ctx, salt_segments **out)
               alloc(&seg->d.blk, (size_t)BLK_INTS * n) && alloc(&seg->d.counts, 4) && alloc(&seg->d.tok_uoff, n) &&
               alloc(&seg->d.tok_urank, n) && alloc(reinterpret_cast<int32_t **>(&seg->d.tok_su), n) &&
               alloc(reinterpret_cast<int32_t **>(&seg->d.tok_sc), n) &&
-              alloc(&seg->d.blk_res, (size_t)n * S_MAX) && alloc(&seg->d.aperm, n) && alloc(&seg->d.a_dptr, n + 1) &&
-              alloc(&seg->d.a_ddom, n) && alloc(&seg->d.a_uptr, n + 1) && alloc(&seg->d.a_udom, n);
+              alloc(&seg->d.blk_res, (size_t)n * S_MAX) && alloc(&seg->d.aperm, n) && alloc(&seg->d.a_uptr, n + 1) &&
+              alloc(&seg->d.a_udom, n) && alloc(&seg->d.u_drun, n) && alloc(&seg->d.d_first, n);
     seg->work.blk_cap = block_bound_loose(ctx, n);
     seg->work.max_group = SALT_MAX_GROUP;
     seg->work.part_cap = PART_CAP;
@@ -938,7 +938,7 @@ void salt_segments_destroy(salt_segments *seg)
                        seg->d.useg_slot, seg->d.blk, seg->d.counts,
                        seg->d.tok_uoff, seg->d.tok_urank, reinterpret_cast<int32_t *>(seg->d.tok_su),
                        reinterpret_cast<int32_t *>(seg->d.tok_sc),
-                       seg->d.blk_res, seg->d.aperm, seg->d.a_dptr, seg->d.a_ddom, seg->d.a_uptr, seg->d.a_udom};
+                       seg->d.blk_res, seg->d.aperm, seg->d.a_uptr, seg->d.a_udom, seg->d.u_drun, seg->d.d_first};
     for (int32_t *p : arrs) cudaFree(p);
     guarded_free(seg->work.vext);
     guarded_free(seg->work.part);

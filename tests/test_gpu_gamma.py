@@ -83,6 +83,17 @@ def test_gamma_segments_host_ids(env, oracle_mod, wl, T):
     assert salt.salt_get_device_error(ctx) == 0
 
 
+@pytest.mark.parametrize("T", [31, 32, 33, 1023, 1024, 1025, 2047, 2049, 16383])
+def test_gamma_segments_sort_edges(env, oracle_mod, wl, T):
+    """The sizes where the sort changes: padded networks up to 1024 keys, then
+    radix passes over one or more rounds of 1024 with a ragged last one."""
+    salt, ctx, seg = env
+    dom, slot, gb = _ids(wl, T, 9, 513, 16, seed=T + 3)
+    salt.salt_build_segments_gamma(ctx, seg, dom, gb, slot, [0.1 * (i + 1) for i in range(16)])
+    _check(salt, ctx, seg, oracle_mod, dom, slot, gb)
+    assert salt.salt_get_device_error(ctx) == 0
+
+
 @pytest.mark.parametrize("T", [300, 16384])
 def test_gamma_segments_device_ids(env, oracle_mod, wl, T):
     salt, ctx, seg = env
