@@ -23,15 +23,16 @@
 //
 // Persistent CTAs over units (tile, K split of KS).  Warp roles:
 //   warp 0      TMA of the W tile (either layout lands as its UMMA descriptor
-//               reads it);
+//               reads it), and of x where a tile's rows are consecutive
+//               tokens;
 //   warp 1      tcgen05.mma into one of two BN-column accumulators;
 //   warps 2-7   everything gathered, by cp.async, a whole stage a warp (six
 //               stages in flight): the token rows of a K chunk, or a delta
 //               chunk's V rows and stacked B rows;
 //   warps 8-11  epilogue: fp32 -> bf16 (RNE) and store, one token row a
-//               thread; with K splits the fp32 partial goes to the workspace
-//               and the split that finishes last sums the tile's partials in
-//               split order (so the result does not depend on timing).
+//               thread; with K splits the fp32 partials go through the
+//               workspace and are summed in split order (so the result does
+//               not depend on timing).
 // The launch is a programmatic dependent of the shrink, which releases it
 // once everything before the shrink is complete: the K loop over x and W
 // overlaps the shrink's tail, and only the delta and the partial stores wait
@@ -66,6 +67,7 @@ struct BaseInfo {
     int32_t ksteps[NST_MAX];               // a delta stage's K = 16 steps
     int32_t mt_b0[MT_MAX], mt_b1[MT_MAX];  // row blocks overlapping M tile: [b0, b1)
     int32_t mt_nd[MT_MAX];                 // its delta chunks
+    int32_t mt_x0[MT_MAX];                 // its first token where this CTA's rows are consecutive tokens, else -1
     uint32_t tmem;
     int32_t last;
 };
@@ -95,6 +97,12 @@ __device__ __forceinline__ void store32(uint16_t *dst, const uint32_t (&w)[8], b
         *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
         *reinterpret_cast<uint4 *>(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
     }
+}
+__device__ __forceinline__ void store_part8(float *dst, const uint32_t *v)
+{
+    asm volatile("st.global.cg.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
 }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
@@ -170,6 +178,19 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             atomicAdd(&info.mt_nd[t], (S + BK - 1) / BK);
         }
     }
+    // Tiles whose rows are consecutive tokens (runs of a prefill batch) take x
+    // by plain TMA tiles; a batch of one tile is not looked at.
+    for (int t = warp; t < n_mt; t += BASE_THREADS / 32) {
+        const int m0 = (t * CG + rank) * BM, rows = min(BM, T - m0);
+        int x0 = -1;
+        if (CG == 2 && rows > 0) {
+            x0 = p.perm[m0];
+            bool lin = true;
+            for (int i = lane; i < rows; i += 32) lin = lin && p.perm[m0 + i] == x0 + i;
+            if (!__all_sync(0xffffffffu, lin)) x0 = -1;
+        }
+        if (lane == 0) info.mt_x0[t] = x0;
+    }
     tc_fence_before();
     cta_or_cluster_sync<CG>();
     tc_fence_after();
@@ -190,22 +211,24 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         bool wrapped = false;  // the ring's first round needs no wait
         auto next_slot = [&]() {
             if (wrapped) wait_bar(info.empty[rp.slot], rp.phase ^ 1u);
+            ok = __all_sync(0xffffffffu, ok);
         };
         auto advance = [&]() {
             rp.advance(1, nst);
             wrapped = wrapped || rp.slot == 0;
         };
-        if (lane == 0) {
-            for (int u = cl; u < n_units && ok; u += n_cl) {
-                const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
-                const int k1 = chunk_lo(s + 1);
-                for (int kc = chunk_lo(s); kc < k1 && ok; ++kc, advance()) {
-                    next_slot();
-                    if (!ok) break;
+        for (int u = cl; u < n_units && ok; u += n_cl) {
+            const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
+            const int k1 = chunk_lo(s + 1), x0 = info.mt_x0[mt];
+            for (int kc = chunk_lo(s); kc < k1 && ok; ++kc, advance()) {
+                next_slot();
+                if (!ok) break;
+                if (elect_one()) {
                     const uint32_t ws = ring32 + rp.slot * stage + x_bytes;
                     const uint32_t fb = leader_addr<CG>(bar(info.full[rp.slot]));
                     const int k0 = kc * BK;
-                    mbar_expect_tx_cluster<CG>(fb, (uint32_t)NB * 128u);
+                    mbar_expect_tx_cluster<CG>(fb, (uint32_t)NB * 128u + (x0 >= 0 ? x_bytes : 0u));
+                    if (x0 >= 0) tma_load_2d_cg<CG>(ws - x_bytes, &p.xmap, k0, x0, fb);
                     if (in_out) {
                         // W[d_in][d_out]: boxes of 64 K rows x 64 N columns (MN-major)
                         for (int h = 0; h < NB / 64; ++h) tma_load_2d_cg<CG>(ws + h * 8192, &p.wmap, n0 + 64 * h, k0, fb);
@@ -214,27 +237,30 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                         tma_load_2d_cg<CG>(ws, &p.wmap, k0, n0, fb);
                     }
                 }
-                // the delta's stages hold nothing of W
-                for (int j = n_delta(mt, s); j > 0 && ok; --j, advance()) {
-                    next_slot();
-                    if (ok) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
-                }
+                __syncwarp();
             }
-            // every stage released (with CG = 2 by the pair's first CTA, whose
-            // arrivals must find this CTA's barriers alive)
-            for (uint32_t i = 0; i < nst; ++i, advance())
-                if (wrapped) wait_bar(info.empty[rp.slot], rp.phase ^ 1u);
+            // the delta's stages hold nothing of W
+            for (int j = n_delta(mt, s); j > 0 && ok; --j, advance()) {
+                next_slot();
+                if (ok && elect_one()) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
+                __syncwarp();
+            }
         }
-        __syncwarp();
+        // every stage released (with CG = 2 by the pair's first CTA, whose
+        // arrivals must find this CTA's barriers alive)
+        for (uint32_t i = 0; i < nst; ++i, advance())
+            if (wrapped) wait_bar(info.empty[rp.slot], rp.phase ^ 1u);
     } else if (warp == 1) {
         // ============================================================ MMA issue
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             const uint32_t id_k = idesc_bf16_f32(BM * CG, BN), id_mn = idesc_bf16_f32_bmn(BM * CG, BN);
             // descriptors of the ring's first stage; a stage adds stage / 16, a
             // K step 2 (K-major: 32 bytes) or 128 (MN-major: 16 rows)
             const uint64_t x0 = sdesc_kmajor_sw128(ring32), wk0 = sdesc_kmajor_sw128(ring32 + x_bytes);
             const uint64_t wmn0 = sdesc_mnmajor_sw128_lbo(ring32 + x_bytes, 8192);
             const uint32_t st16 = stage >> 4;
+            const uint64_t w0 = in_out ? wmn0 : wk0;
+            const uint32_t w_step = in_out ? 128 : 2, id_w = in_out ? id_mn : id_k;
             RingPos rp;
             uint32_t lt = 0;
             for (int u = cl; u < n_units; u += n_cl, ++lt) {
@@ -246,36 +272,32 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                 for (int n = chunk_lo(s + 1) - chunk_lo(s); n > 0; --n, rp.advance(1, nst)) {
                     wait_bar(info.full[rp.slot], rp.phase);
                     tc_fence_after();
-                    const uint64_t xd = x0 + rp.slot * st16;
-                    if (in_out) {
-                        const uint64_t wd = wmn0 + rp.slot * st16;
+                    const uint64_t xd = x0 + rp.slot * st16, wd = w0 + rp.slot * st16;
+                    if (elect_one()) {
 #pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-                            umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, accum);
-                            accum = 1;
-                        }
-                    } else {
-                        const uint64_t wd = wk0 + rp.slot * st16;
-#pragma unroll
-                        for (int kk = 0; kk < BK / 16; ++kk) {
-                            umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 2, id_k, accum);
-                            accum = 1;
-                        }
+                        for (int kk = 0; kk < BK / 16; ++kk)
+                            umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * w_step, id_w, kk > 0 ? 1u : accum);
+                        umma_commit_cg<CG>(bar(info.empty[rp.slot]));
                     }
-                    umma_commit_cg<CG>(bar(info.empty[rp.slot]));
+                    __syncwarp();
+                    accum = 1;
                 }
                 for (int n = n_delta(mt, s); n > 0; --n, rp.advance(1, nst)) {
                     wait_bar(info.full[rp.slot], rp.phase);
                     tc_fence_after();
                     const uint64_t xd = x0 + rp.slot * st16, wd = wmn0 + rp.slot * st16;
+                    ok = __all_sync(0xffffffffu, ok);
                     const int steps = ok ? *reinterpret_cast<volatile int32_t *>(&info.ksteps[rp.slot]) : 0;
-                    for (int kk = 0; kk < steps; ++kk) {
-                        umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, accum);
-                        accum = 1;
+                    if (elect_one()) {
+                        for (int kk = 0; kk < steps; ++kk)
+                            umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, kk > 0 ? 1u : accum);
+                        umma_commit_cg<CG>(bar(info.empty[rp.slot]));
                     }
-                    umma_commit_cg<CG>(bar(info.empty[rp.slot]));
+                    __syncwarp();
+                    accum = 1;
                 }
-                umma_commit_cg<CG>(bar(info.accf[buf]));
+                if (elect_one()) umma_commit_cg<CG>(bar(info.accf[buf]));
+                __syncwarp();
             }
         }
         __syncwarp();
@@ -291,16 +313,19 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             if (wrapped) wait_bar(info.empty[rp.slot], rp.phase ^ 1u);
             ok = __all_sync(0xffffffffu, ok);
         };
+        auto next_stage = [&]() {
+            const uint32_t before = rp.slot;
+            rp.advance(GWN, nst);
+            wrapped = wrapped || rp.slot <= before;
+            mine += GWN;
+        };
         auto finish = [&]() {       // the warp's copies have landed; on to its next stage
             cp_async_commit();
             cp_async_wait<0>();
             fence_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
-            const uint32_t before = rp.slot;
-            rp.advance(GWN, nst);
-            wrapped = wrapped || rp.slot <= before;
-            mine += GWN;
+            next_stage();
         };
         uint32_t xoff[BM / 4];      // this lane's token rows (row 4 i + lane / 8), in 16-byte units of x
         int mt_of = -1, rows = 0;
@@ -308,7 +333,8 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         for (int u = cl; u < n_units && ok; u += n_cl) {
             const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
             const int m0 = (mt * CG + rank) * BM;
-            if (mt != mt_of) {
+            const bool lin = info.mt_x0[mt] >= 0;
+            if (mt != mt_of && !lin) {
                 mt_of = mt;
                 rows = max(0, min(BM, T - m0));
 #pragma unroll
@@ -324,6 +350,11 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             while ((int)mine < n && ok) {
                 begin();
                 if (!ok) break;
+                if (lin) {  // the TMA warp loads the rows
+                    if (lane == 0) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
+                    next_stage();
+                    continue;
+                }
                 const int kc = k0 + (int)mine;
                 const uint32_t xs = ring32 + rp.slot * stage;
                 const bool in = kc * BK + (lane & 7) * 8 < p.d_in;
@@ -406,6 +437,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         const int q = warp & 3, row = q * 32 + lane, et = tid - 32 * EW0;
         const bool wide = (p.d_out & 15) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 31) == 0;
         uint32_t lt = 0;
+        const bool share = n_units <= n_cl;
         if (KS > 1) pdl_wait();  // the partials' workspace is the shrink's
         for (int u = cl; u < n_units; u += n_cl, ++lt) {
             const int tile = u / KS, mt = tile % n_mt, n0 = tile / n_mt * BN;
@@ -429,12 +461,10 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     for (int h = 0; h < 2; ++h) {
                         const int col = n0 + c + 16 * h;
                         if (tok < 0) continue;
-                        if (KS > 1) {
-                            float4 *dst = reinterpret_cast<float4 *>(part + row * BN + c + 16 * h);
+                        if (KS > 1) {  // [8 columns][row][8]: a warp's stores are contiguous
 #pragma unroll
-                            for (int i = 0; i < 4; ++i)
-                                __stcg(dst + i, make_float4(__uint_as_float(v[h][4 * i]), __uint_as_float(v[h][4 * i + 1]),
-                                                            __uint_as_float(v[h][4 * i + 2]), __uint_as_float(v[h][4 * i + 3])));
+                            for (int i = 0; i < 2; ++i)
+                                store_part8(part + ((c >> 3) + 2 * h + i) * (m_rows * 8) + row * 8, v[h] + 8 * i);
                             continue;
                         }
                         uint32_t w[8];
@@ -450,23 +480,39 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             __syncwarp();
             if (lane == 0) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.acce[buf])));
             if (KS == 1) continue;
-            // the split that finishes the tile last (this CTA's rows) sums its partials
+            // Sum the partials of the tile (this CTA's rows) in split order.
+            // When every unit has its own CTAs at once, each split waits
+            // (bounded) for the others and sums its share; otherwise the
+            // split that finishes last sums them all.
             __threadfence();
             named_sync(BAR_E, EPI_N);
+            uint32_t *ctr = p.ctr + 2 * (tile * CG + rank);
             if (et == 0) {
-                uint32_t *ctr = p.ctr + (tile * CG + rank);
-                const uint32_t n = atomicAdd(ctr, 1u);
-                info.last = n == (uint32_t)KS - 1u;
-                if (info.last) atomicExch(ctr, 0u);  // zero for the next launch
+                const uint32_t n = atomicAdd(ctr, 1u) + 1u;
+                bool go = n == (uint32_t)KS;
+                if (share) {
+                    for (int i = 0; i < (1 << 22) && !go; ++i) {
+                        uint32_t c;
+                        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(c) : "l"(ctr) : "memory");
+                        go = c == (uint32_t)KS;
+                        if (!go) __nanosleep(32);
+                    }
+                    if (!go) ok = false;
+                    go = true;
+                } else if (go) {
+                    atomicExch(ctr, 0u);  // zero for the next launch
+                }
+                info.last = go;
                 __threadfence();
             }
             named_sync(BAR_E, EPI_N);
             if (!info.last) continue;
             const float *p0 = p.part + ((int64_t)tile * KS * CG + rank) * (m_rows * BN);
             const int64_t ps = (int64_t)CG * m_rows * BN;
-            const int cpr = BN >> 3, n_it = rows * cpr;
+            const int lc = BN == 256 ? 5 : 4, n_all = rows << lc, s_own = u - tile * KS;
+            const int n_it = share ? n_all * (s_own + 1) / KS : n_all;
             // (row, 8 columns) items, two a round per thread, up to four splits' loads in flight
-            for (int base = et; base < n_it; base += 2 * EPI_N) {
+            for (int base = (share ? n_all * s_own / KS : 0) + et; base < n_it; base += 2 * EPI_N) {
                 float a[2][8] = {};
                 for (int s0 = 0; s0 < KS; s0 += 4) {
                     float4 v[2][4][2];
@@ -476,7 +522,8 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                         for (int s = 0; s < 4; ++s) {
                             const int it = base + h * EPI_N;
                             if (it < n_it && s0 + s < KS) {
-                                const float4 *src = reinterpret_cast<const float4 *>(p0 + (s0 + s) * ps + (int64_t)it * 8);
+                                const int c8 = it & ((1 << lc) - 1), r = it >> lc;
+                                const float4 *src = reinterpret_cast<const float4 *>(p0 + (s0 + s) * ps + (c8 * m_rows + r) * 8);
                                 v[h][s][0] = __ldcg(src);
                                 v[h][s][1] = __ldcg(src + 1);
                             } else {
@@ -501,11 +548,19 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                 for (int h = 0; h < 2; ++h) {
                     const int it = base + h * EPI_N;
                     if (it >= n_it) continue;
-                    const int r = it / cpr, col = n0 + (it - r * cpr) * 8;
+                    const int r = it >> lc, col = n0 + (it & ((1 << lc) - 1)) * 8;
                     if (col < p.d_out)
                         *reinterpret_cast<uint4 *>(p.y + (int64_t)p.perm[m0 + r] * p.d_out + col) =
                             make_uint4(pack_bf16(a[h][0], a[h][1]), pack_bf16(a[h][2], a[h][3]),
                                        pack_bf16(a[h][4], a[h][5]), pack_bf16(a[h][6], a[h][7]));
+                }
+            }
+            if (share) {
+                // the last split to have read the partials zeroes the counters
+                named_sync(BAR_E, EPI_N);
+                if (et == 0 && atomicAdd(ctr + 1, 1u) + 1u == (uint32_t)KS) {
+                    atomicExch(ctr, 0u);
+                    atomicExch(ctr + 1, 0u);
                 }
             }
         }
@@ -521,7 +576,8 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     if (warp == 1) tmem_dealloc<CG>(tmem, 2 * BN);
 }
 
-int g_base_sms[64];
+int g_base_sms[64];    // SMs per device, and the CTA pairs that fit on them at once (filled by base_prepare)
+int g_base_pairs[64];
 
 struct BasePlan {
     int cg, bn, ks;
@@ -531,9 +587,9 @@ struct BasePlan {
 // cycles: whole waves of units over the SMs (pairs of SMs for CG = 2), a
 // chunk's cost, a fixed cost per wave and, with splits, the partials' way
 // through L2.
-BasePlan base_plan(int T, int d_in, int d_out, int n_sm, int part_floats)
+BasePlan base_plan(int T, int d_in, int d_out, int n_sm, int n_pairs, int part_floats)
 {
-    const int nk = (d_in + BK - 1) / BK, cg = T > BM ? 2 : 1, n_cl = std::max(1, n_sm / cg);
+    const int nk = (d_in + BK - 1) / BK, cg = T > BM ? 2 : 1, n_cl = std::max(1, cg == 2 ? n_pairs : n_sm);
     const int n_mt = (T + BM * cg - 1) / (BM * cg), m_rows = cg == 2 ? BM : (std::min(T, BM) + 15) & ~15;
     BasePlan best = {cg, 128, 1};
     double best_cost = 1e30;
@@ -541,7 +597,7 @@ BasePlan base_plan(int T, int d_in, int d_out, int n_sm, int part_floats)
         const int n_nt = (d_out + bn - 1) / bn;
         for (int ks = 1; ks <= std::min(BASE_KS_MAX, nk); ++ks) {
             const int64_t tiles = (int64_t)n_mt * n_nt, units = tiles * ks;
-            if (ks > 1 && (units * cg * m_rows * bn > part_floats || tiles * cg > BASE_CTRS)) break;
+            if (ks > 1 && (units * cg * m_rows * bn > part_floats || 2 * tiles * cg > BASE_CTRS)) break;
             const double waves = (double)((units + n_cl - 1) / n_cl);
             const double chunk = cg == 2 ? (bn == 256 ? 560 : 340) : 600;
             const double split = ks > 1 ? (double)m_rows * bn * (0.06 + 0.06 * ks) + 3000 : 0;
@@ -564,7 +620,20 @@ cudaError_t base_prepare(int device)
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(salt_base_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BASE_SMEM);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(salt_base_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BASE_SMEM);
+    e = cudaFuncSetAttribute(salt_base_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BASE_SMEM);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((g_base_sms[device] & ~1) > 0 ? g_base_sms[device] & ~1 : 2, 1, 1);
+    cfg.blockDim = dim3(BASE_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = BASE_SMEM;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(&g_base_pairs[device], salt_base_kernel<2>, &cfg);
 }
 
 cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream)
@@ -573,7 +642,8 @@ cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const int n_sm = (dev >= 0 && dev < 64 && g_base_sms[dev] > 0) ? g_base_sms[dev] : 1;
-    BasePlan pl = base_plan(p.T, p.d_in, p.d_out, n_sm, PART_CAP * TM * PART_COLS);
+    const int n_pairs = (dev >= 0 && dev < 64) ? g_base_pairs[dev] : 0;
+    const BasePlan pl = base_plan(p.T, p.d_in, p.d_out, n_sm, n_pairs, PART_CAP * TM * PART_COLS);
     p.bn = pl.bn;
     p.ks = pl.ks;
     const cuuint32_t nb = (cuuint32_t)(pl.bn / pl.cg);
@@ -581,10 +651,11 @@ cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream)
     // W_base[d_out][d_in]: NB rows x 64 K
     e = p.w_layout == SALT_W_IN_OUT ? encode_map_2d(&p.wmap, W, p.d_out, p.d_in, 64, 64)
                                     : encode_map_2d(&p.wmap, W, p.d_in, p.d_out, 64, nb);
+    if (e == cudaSuccess) e = encode_map_2d(&p.xmap, p.x, p.d_in, p.T, 64, BM);
     if (e != cudaSuccess) return e;
     const int bm = BM * pl.cg;
     const int64_t units = (int64_t)((p.T + bm - 1) / bm) * ((p.d_out + pl.bn - 1) / pl.bn) * pl.ks;
-    const int n_cl = (int)std::min<int64_t>(units, std::max(1, n_sm / pl.cg));
+    const int n_cl = (int)std::min<int64_t>(units, std::max(1, pl.cg == 2 ? n_pairs : n_sm));
     if (n_cl <= 0) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];

@@ -171,6 +171,7 @@ struct BaseParams {
     // 64 (N) x 64 (K), for SALT_W_OUT_IN the tensor [d_out][d_in] with box
     // 64 (K) x the W columns a CTA loads
     alignas(64) CUtensorMap wmap;
+    alignas(64) CUtensorMap xmap;  // x [T][d_in], box 64 x 128 tokens
     const uint16_t *x;       // [T][d_in]
     uint16_t *y;             // [T][d_out], written
     const int32_t *perm;     // grouped position -> token
@@ -183,7 +184,7 @@ struct BaseParams {
     int64_t slot_stride;
     int64_t res_off;         // sum over earlier layers of (d_in + d_out), in elements
     float *part;             // fp32 partials of the K splits (the apply's partial tiles)
-    uint32_t *ctr;           // [BASE_CTRS] splits finished, per (tile, CTA of the pair); zero between launches
+    uint32_t *ctr;           // [BASE_CTRS] splits stored and summed, per (tile, CTA of the pair); zero between launches
     int32_t T, d_in, d_out, rc_max, w_layout, blk_cap;
     int32_t bn, ks;          // tile columns and K splits (launch_base)
     uint32_t *err;

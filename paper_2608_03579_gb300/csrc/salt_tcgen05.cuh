@@ -36,6 +36,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     return false;
 }
 
+// One thread of a converged warp, the same each time.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
+
 // ---------------------------------------------------------------- TMEM
 // Allocate ncols (power of two, >= 32) tensor-memory columns; one whole warp
 // executes it; the TMEM address lands in shared memory at dst.
@@ -166,14 +174,16 @@ __device__ __forceinline__ void cta_or_cluster_sync()
     }
 }
 // Arrivals on a barrier of either CTA of the pair (an address of
-// leader_addr).  A cluster-scope release in the thread that feeds every
-// stage was measured at 0.4 us a stage, so the TMA thread arrives relaxed:
-// what its stages guard is ordered by the copies' own completion.
+// leader_addr).  What a stage guards lies in the arriving thread's own CTA
+// and is read there by the tensor core (the async proxy, after the thread's
+// fence.proxy.async), so CTA scope is what the release has to cover; a
+// cluster-scope release waits for the thread's other traffic too and cost
+// 0.4 us a stage in the TMA thread and 0.1 us in the gather warps.
 template <int CG>
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar)
 {
     if (CG == 1) asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-    else asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
+    else asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 template <int CG>
 __device__ __forceinline__ void mbar_arrive_relaxed_cluster(uint32_t bar)
