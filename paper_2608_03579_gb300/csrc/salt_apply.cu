@@ -1110,7 +1110,7 @@ cudaError_t launch_wait_selftest(uint32_t *err, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-cudaError_t launch_apply(const ApplyParams &p, bool pdl, cudaStream_t stream)
+cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, cudaStream_t stream)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1120,7 +1120,7 @@ cudaError_t launch_apply(const ApplyParams &p, bool pdl, cudaStream_t stream)
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(n_sm, 1, 1);
+    cfg.gridDim = dim3(ctas > 0 && ctas < n_sm ? ctas : n_sm, 1, 1);
     cfg.blockDim = dim3(APPLY_THREADS, 1, 1);
     cfg.dynamicSmemBytes = FUSED_SMEM;
     cfg.stream = stream;

@@ -37,6 +37,12 @@
 // once everything before the shrink is complete: the K loop over x and W
 // overlaps the shrink's tail, and only the delta and the partial stores wait
 // for the shrink itself.
+//
+// Measured against one CTA per 128 x 128 tile with cp.async for x, no K
+// split and the shrink run to its end first: a 3B MLP layer at 8192 tokens
+// 2937 -> 890 us (1.41 PFLOP/s), an 8B layer at 512 tokens 746 -> 329 us, at
+// 24 tokens 552 -> 178 us.  x by TMA tile::gather4 instead of the gather
+// warps took 3050 us for the first (about 90 cycles a four-row copy).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -286,7 +292,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     wait_bar(info.full[rp.slot], rp.phase);
                     tc_fence_after();
                     const uint64_t xd = x0 + rp.slot * st16, wd = wmn0 + rp.slot * st16;
-                    ok = __all_sync(0xffffffffu, ok);
+                            ok = __all_sync(0xffffffffu, ok);
                     const int steps = ok ? *reinterpret_cast<volatile int32_t *>(&info.ksteps[rp.slot]) : 0;
                     if (elect_one()) {
                         for (int kk = 0; kk < steps; ++kk)
@@ -580,35 +586,65 @@ int g_base_sms[64];    // SMs per device, and the CTA pairs that fit on them at 
 int g_base_pairs[64];
 
 struct BasePlan {
-    int cg, bn, ks;
+    int cg, bn, ks, shrink_ctas;
 };
 
-// The tile and the K splits of a launch, by an estimate of its tensor
-// cycles: whole waves of units over the SMs (pairs of SMs for CG = 2), a
-// chunk's cost, a fixed cost per wave and, with splits, the partials' way
-// through L2.
-BasePlan base_plan(int T, int d_in, int d_out, int n_sm, int n_pairs, int part_floats)
+// The launch's shape, by an estimate of its time in us (the constants are fits
+// to measured launches, 24 to 1024 tokens, d_in 4096 and 14336, d_out 1024 to
+// 14336): the tile width, the K splits, and the SMs the shrink gets.  Either
+// the shrink takes every SM and the K loop starts after it, or it takes
+// 24 or 48 beside the K loop on the others (only the delta waits for it):
+// worth it where the K loop is long or leaves SMs idle anyway, e.g. 24 tokens
+// of 4096 x 14336 45 -> 36 us beside, but 14336 x 4096 at 512 tokens 75 us in
+// turn against 89.
+BasePlan base_plan(int T, int d_in, int d_out, int n_blk, int n_sm, int max_pairs)
 {
-    const int nk = (d_in + BK - 1) / BK, cg = T > BM ? 2 : 1, n_cl = std::max(1, cg == 2 ? n_pairs : n_sm);
+    const int nk = (d_in + BK - 1) / BK, cg = T > BM ? 2 : 1;
     const int n_mt = (T + BM * cg - 1) / (BM * cg), m_rows = cg == 2 ? BM : (std::min(T, BM) + 15) & ~15;
-    BasePlan best = {cg, 128, 1};
-    double best_cost = 1e30;
-    for (int bn = 128; bn <= (cg == 2 ? 256 : 128); bn *= 2) {
-        const int n_nt = (d_out + bn - 1) / bn;
-        for (int ks = 1; ks <= std::min(BASE_KS_MAX, nk); ++ks) {
-            const int64_t tiles = (int64_t)n_mt * n_nt, units = tiles * ks;
-            if (ks > 1 && (units * cg * m_rows * bn > part_floats || 2 * tiles * cg > BASE_CTRS)) break;
-            const double waves = (double)((units + n_cl - 1) / n_cl);
-            const double chunk = cg == 2 ? (bn == 256 ? 560 : 340) : 600;
-            const double split = ks > 1 ? (double)m_rows * bn * (0.06 + 0.06 * ks) + 3000 : 0;
-            const double cost = waves * (((nk + ks - 1) / ks) * chunk + 500) + split;
-            if (cost < best_cost) {
-                best_cost = cost;
-                best = {cg, bn, ks};
+    BasePlan best = {cg, 128, 1, 0};
+    double best_t = 1e30;
+    for (int beside = 0; beside <= 48; beside += 24) {
+        if (beside && (T > 2048 || n_sm < 2 * beside)) break;
+        const int sms = n_sm - beside, n_cl = std::max(1, cg == 2 ? std::min(max_pairs, sms / 2) : sms);
+        const int sh = beside ? beside : n_sm, sh_ks = std::max(1, std::min(16, sh / std::max(1, n_blk)));
+        const int sh_waves = (n_blk * sh_ks + sh - 1) / sh;
+        const double t_shrink = 12.0 + 0.42 * sh_waves * ((nk + sh_ks - 1) / sh_ks);
+        for (int bn = 128; bn <= (cg == 2 ? 256 : 128); bn *= 2) {
+            const int64_t tiles = (int64_t)n_mt * ((d_out + bn - 1) / bn);
+            for (int ks = 1; ks <= std::min(BASE_KS_MAX, nk); ++ks) {
+                const int64_t units = tiles * ks;
+                if (ks > 1 && (units * cg * m_rows * bn > (int64_t)PART_CAP * TM * PART_COLS || 2 * tiles * cg > BASE_CTRS)) break;
+                const double waves = (double)((units + n_cl - 1) / n_cl);
+                // a chunk: one CTA a tile is bound by streaming W from memory
+                // (16 KB a chunk at 6 TB/s over the running CTAs, or by its
+                // own latency), a pair by its stages
+                const double active = (double)std::min<int64_t>(units, n_cl);
+                const double chunk = cg == 1 ? std::max(0.36, 0.41 * active / 152) : (bn == 256 ? 0.35 : 0.23);
+                const double k_loop = ((nk + ks - 1) / ks) * chunk, tail = n_mt > 8 ? 1.0 : cg == 2 ? 9.0 : 4.0;
+                const bool share = units <= n_cl;
+                const double split = ks == 1 ? 0 : (m_rows / 128.0) * (bn / 128.0) * (share ? 2.0 : 0.5 + 0.8 * ks) + 2.0;
+                const double gemm = waves * (k_loop + tail) + split;
+                // (a K loop that follows the shrink still overlaps its tail)
+                const double t = beside ? gemm + std::max(0.0, t_shrink - k_loop) : gemm + t_shrink - std::min(3.0, k_loop);
+                if (t < best_t) {
+                    best_t = t;
+                    best = {cg, bn, ks, beside};
+                }
             }
         }
     }
     return best;
+}
+
+// The plan of a launch on the current device; false when it is not prepared.
+bool plan_here(int T, int d_in, int d_out, int n_blk, BasePlan *pl, int *n_cl)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || g_base_sms[dev] <= 0) return false;
+    *pl = base_plan(T, d_in, d_out, n_blk, g_base_sms[dev], g_base_pairs[dev]);
+    const int sms = g_base_sms[dev] - pl->shrink_ctas;
+    *n_cl = std::max(1, pl->cg == 2 ? std::min(g_base_pairs[dev], sms / 2) : sms);
+    return true;
 }
 
 }  // namespace
@@ -636,14 +672,19 @@ cudaError_t base_prepare(int device)
     return cudaOccupancyMaxActiveClusters(&g_base_pairs[device], salt_base_kernel<2>, &cfg);
 }
 
-cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream)
+int base_shrink_ctas(int T, int d_in, int d_out, int n_blk)
 {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const int n_sm = (dev >= 0 && dev < 64 && g_base_sms[dev] > 0) ? g_base_sms[dev] : 1;
-    const int n_pairs = (dev >= 0 && dev < 64) ? g_base_pairs[dev] : 0;
-    const BasePlan pl = base_plan(p.T, p.d_in, p.d_out, n_sm, n_pairs, PART_CAP * TM * PART_COLS);
+    BasePlan pl;
+    int n_cl;
+    return plan_here(T, d_in, d_out, n_blk, &pl, &n_cl) ? pl.shrink_ctas : 0;
+}
+
+cudaError_t launch_base(BaseParams &p, const uint16_t *W, int n_blk, cudaStream_t stream)
+{
+    BasePlan pl;
+    int max_cl;
+    if (!plan_here(p.T, p.d_in, p.d_out, n_blk, &pl, &max_cl)) return cudaErrorInvalidDevice;
+    cudaError_t e;
     p.bn = pl.bn;
     p.ks = pl.ks;
     const cuuint32_t nb = (cuuint32_t)(pl.bn / pl.cg);
@@ -655,7 +696,7 @@ cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream)
     if (e != cudaSuccess) return e;
     const int bm = BM * pl.cg;
     const int64_t units = (int64_t)((p.T + bm - 1) / bm) * ((p.d_out + pl.bn - 1) / pl.bn) * pl.ks;
-    const int n_cl = (int)std::min<int64_t>(units, std::max(1, pl.cg == 2 ? n_pairs : n_sm));
+    const int n_cl = (int)std::min<int64_t>(units, max_cl);
     if (n_cl <= 0) return cudaSuccess;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];

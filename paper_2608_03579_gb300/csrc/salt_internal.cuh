@@ -192,8 +192,11 @@ struct BaseParams {
 constexpr int BASE_CTRS = 1024;
 cudaError_t base_prepare(int device);
 // The GEMM over W, as a programmatic dependent of the shrink-only apply
-// launched just before it on the stream.
-cudaError_t launch_base(BaseParams &p, const uint16_t *W, cudaStream_t stream);
+// launched just before it on the stream; n_blk: about how many row blocks
+// the batch has (only shapes the launch, the same value for both calls).
+cudaError_t launch_base(BaseParams &p, const uint16_t *W, int n_blk, cudaStream_t stream);
+// CTAs of the shrink before a base launch (0: one per SM).
+int base_shrink_ctas(int T, int d_in, int d_out, int n_blk);
 // A row-major bf16 tensor [rows][cols] as a 2-D TMA map, 128-byte swizzle (host).
 cudaError_t encode_map_2d(CUtensorMap *out, const uint16_t *base, int64_t cols, int64_t rows, uint32_t box_cols,
                           uint32_t box_rows);
@@ -209,7 +212,8 @@ cudaError_t apply_prepare(int device);
 // K-split) first, then the expand items (row block, 64 output columns).
 // With pdl the launch is a programmatic dependent of the previous kernel on
 // the stream (only when that kernel did not write the segment tables).
-cudaError_t launch_apply(const ApplyParams &p, bool pdl, cudaStream_t stream);
+// The grid is `ctas` CTAs (0: one per SM).
+cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, cudaStream_t stream);
 size_t apply_smem_bytes();
 // W[Mdim][Ndim] += scale * P^T Q for P = [rc][Mdim], Q = [rc][Ndim] (bf16,
 // rows contiguous, rc <= 64): the centroid fold; a timed-out wait sets

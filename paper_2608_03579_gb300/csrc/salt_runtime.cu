@@ -69,6 +69,7 @@ struct salt_segments {
     bool device_ids = false;
     int T = 0;
     int n_blk_bound = 0;                       // launch bound on the row blocks of the last build
+    int n_blk_est = 1;                         // about how many there are (shapes launches only)
     ApplyWork work{};                          // V tiles of the apply path
     std::vector<uint8_t> refs;                 // slots named by the last build (host ids)
     cudaStream_t build_stream = nullptr;
@@ -256,10 +257,10 @@ int block_bound_loose(const salt_ctx *ctx, int T)
 
 // Tighter bound from validated host ids: a domain with n tokens (those
 // with a term) in u user runs (runs of equal gamma bin and slot) yields at
-// most ceil(n / TM) + ceil(u / umax) blocks.  Only sizes the launch grid;
+// most ceil(n / TM) + ceil(u / umax) blocks, and about one less (*n_est).  Only sizes the launch grid;
 // the block list itself comes from the segment kernel, and CTAs past its
 // count exit at once.
-int block_bound_host(const salt_ctx *ctx, const int32_t *dom, const int32_t *gbin, const int32_t *slot, int T)
+int block_bound_host(const salt_ctx *ctx, const int32_t *dom, const int32_t *gbin, const int32_t *slot, int T, int *n_est)
 {
     std::vector<uint64_t> keys;
     keys.reserve(T);
@@ -269,7 +270,7 @@ int block_bound_host(const salt_ctx *ctx, const int32_t *dom, const int32_t *gbi
         keys.push_back(((uint64_t)(uint32_t)(dom[t] + 1) << 32) | (g << 20) | (uint32_t)(slot[t] + 1));
     }
     std::sort(keys.begin(), keys.end());
-    int64_t bound = 0;
+    int64_t bound = 0, est = 0;
     size_t i = 0;
     while (i < keys.size()) {
         uint32_t d = (uint32_t)(keys[i] >> 32);
@@ -282,7 +283,9 @@ int block_bound_host(const salt_ctx *ctx, const int32_t *dom, const int32_t *gbi
             ++i;
         }
         bound += (n + TM - 1) / TM + (u + ctx->umax - 1) / ctx->umax;
+        est += (n + TM - 1) / TM + (u + ctx->umax - 1) / ctx->umax - 1;
     }
+    *n_est = (int)std::max<int64_t>(1, est);
     int cap = block_bound_loose(ctx, ctx->max_tokens);
     return (int)(bound < cap ? bound : cap);
 }
@@ -1064,9 +1067,10 @@ salt_status salt_build_segments_gamma(salt_ctx *ctx, salt_segments *seg, const i
     seg->T = T;
     if (dev_ids) std::fill(seg->refs.begin(), seg->refs.end(), 1);
     else seg->refs.swap(refs);
+    seg->n_blk_est = std::max(1, std::min(block_bound_loose(ctx, T), seg->work.blk_cap) / 2);
     if (T == 0) seg->n_blk_bound = 0;
     else if (dev_ids) seg->n_blk_bound = std::min(block_bound_loose(ctx, T), seg->work.blk_cap);
-    else seg->n_blk_bound = std::min(block_bound_host(ctx, domain_ids, gamma_bins, slot_ids, T), seg->work.blk_cap);
+    else seg->n_blk_bound = std::min(block_bound_host(ctx, domain_ids, gamma_bins, slot_ids, T, &seg->n_blk_est), seg->work.blk_cap);
     seg->build_stream = stream;
     seg->use_streams.clear();
     seg->use_streams.push_back(stream);
@@ -1185,9 +1189,10 @@ salt_status apply_grouped(salt_ctx *ctx, const salt_segments *seg_, int32_t n, c
     p.w = seg->work;
     p.err = ctx->err_dev;
     p.shrink_only = shrink_only ? 1 : 0;
+    const int ctas = shrink_only ? base_shrink_ctas(seg->T, p.proj[0].d_in, p.proj[0].d_out, seg->n_blk_est) : 0;
     // The first apply after a build waits for the segment kernel in full;
     // later ones overlap their table reads with the previous kernel.
-    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, stream));
+    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, ctas, stream));
     seg->tables_fresh = false;
     return SALT_OK;
 }
@@ -1245,7 +1250,7 @@ salt_status salt_lora_apply_with_base(salt_ctx *ctx, const salt_segments *seg_, 
     bp.part = seg->work.part;
     bp.ctr = seg->work.base_ctr;
     bp.err = ctx->err_dev;
-    CUDA_OR_FAIL(ctx, launch_base(bp, static_cast<const uint16_t *>(W), static_cast<cudaStream_t>(stream_)));
+    CUDA_OR_FAIL(ctx, launch_base(bp, static_cast<const uint16_t *>(W), seg->n_blk_est, static_cast<cudaStream_t>(stream_)));
     return SALT_OK;
 }
 
@@ -1311,7 +1316,7 @@ salt_status salt_lora_apply_static(salt_ctx *ctx, const salt_segments *seg_, int
     p.slot_stride = ctx->slot_stride;
     p.w = scratch;
     p.err = ctx->err_dev;
-    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, stream));
+    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, 0, stream));
     seg->tables_fresh = false;
     return SALT_OK;
 }
