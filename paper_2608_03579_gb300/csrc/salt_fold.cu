@@ -23,11 +23,17 @@
 //              into one of four accumulators;
 //   warp 2     P^T of each row tile into a K-major swizzled A tile (two
 //              buffers), an 8 x 8 register transpose per 16-byte chunk;
-//   warps 3-6  the epilogue, one W row a thread: scale * D added to the W
-//              tile in shared memory in fp32, rounded once to bf16, and the
-//              tile written back by a TMA store; the stage is released once
-//              the store has read it.
+//   warps 3-10 the epilogue, two groups of four warps taking items in turn,
+//              one W row a thread: scale * D added to the W tile in shared
+//              memory in fp32, rounded once to bf16, and the tile written back
+//              by a TMA store; the stage is released once the store has read
+//              it.
 // Rows >= Mdim and columns >= Ndim are zero on load and clipped on store.
+//
+// Bound by reading and writing W: two 8B layers (1.77 GB moved) go at 6.07
+// TB/s (a plain copy: 6.8).  One epilogue group that found each item's place
+// by 64-bit division and table reads was the bound before: two 8B layers in
+// a plan 363 -> 291 us, one 3072 x 3072 weight 10.1 -> 7.1 us.
 #include "salt_async.cuh"
 #include "salt_internal.cuh"
 #include "salt_pipe.cuh"
@@ -39,7 +45,7 @@
 namespace salt {
 namespace {
 
-constexpr int FOLD_THREADS = 224;
+constexpr int FOLD_THREADS = 352;
 constexpr int FOLD_TM = 128;                          // W rows per tile (UMMA M)
 constexpr int FOLD_NC = 64;                           // W columns per item (UMMA N)
 constexpr int FOLD_STAGES = 7;
@@ -50,10 +56,12 @@ constexpr int FOLD_STAGE_BYTES = FOLD_W_BYTES + FOLD_Q_BYTES;
 constexpr int FOLD_A_BYTES = FOLD_TM * 128;           // [128 rows][K <= 64], K-major
 constexpr int FOLD_SMEM = 1024 + 2 * FOLD_A_BYTES + FOLD_STAGES * FOLD_STAGE_BYTES;
 constexpr int FOLD_EPI_WARP0 = 3;
-constexpr int FOLD_EPI_THREADS = 128;
-constexpr int FOLD_BAR_EPI = 1;                       // named barrier of the epilogue warps
+constexpr int FOLD_EPI_THREADS = 128;                 // of one epilogue group
+constexpr int FOLD_EPI_GROUPS = 2;                    // items j, j + 1 in turn
+constexpr int FOLD_BAR_EPI = 1;                       // named barriers of the epilogue groups (1, 2)
 static_assert(FOLD_SMEM <= 227 * 1024, "fold shared memory");
-static_assert(FOLD_THREADS == 32 * FOLD_EPI_WARP0 + FOLD_EPI_THREADS, "warp roles");
+static_assert(FOLD_THREADS == 32 * FOLD_EPI_WARP0 + FOLD_EPI_GROUPS * FOLD_EPI_THREADS, "warp roles");
+static_assert(FOLD_NACC % FOLD_EPI_GROUPS == 0, "an accumulator belongs to one epilogue group");
 static_assert(SALT_MAX_CENTROID_RANK <= 64, "K of the fold is one 128-byte row");
 
 // One weight of a fold launch.  In a plan's device table the records lie
@@ -86,10 +94,34 @@ __device__ __forceinline__ int fold_find(const FoldMat *M, int nm, int64_t it)
     }
     return lo;
 }
-__device__ __forceinline__ void fold_advance(const FoldMat *M, int nm, int64_t it, int &mat)
-{
-    while (mat + 1 < nm && it >= M[mat + 1].item0) ++mat;
-}
+// A CTA's place in the items, stepped one at a time: nothing is divided and
+// no table entry read but at a new weight.
+struct FoldCursor {
+    const FoldMat *F;
+    int rt, ct, n_rt, n_ct;  // row tile and 64-column item, and how many of each
+    __device__ void load(const FoldMat *f)
+    {
+        F = f;
+        n_rt = (f->Mdim + FOLD_TM - 1) / FOLD_TM;
+        n_ct = (f->Ndim + FOLD_NC - 1) / FOLD_NC;
+    }
+    __device__ void start(const FoldMat *M, int nm, int64_t it)
+    {
+        load(M + fold_find(M, nm, it));
+        rt = (int)((it - F->item0) / n_ct);
+        ct = (int)((it - F->item0) - (int64_t)rt * n_ct);
+    }
+    __device__ bool ends_tile() const { return ct + 1 == n_ct; }
+    // to the next item (which must exist)
+    __device__ void step()
+    {
+        if (++ct < n_ct) return;
+        ct = 0;
+        if (++rt < n_rt) return;
+        rt = 0;
+        load(F + 1);
+    }
+};
 // a table map written by the host is read by the TMA unit through the
 // tensor-map proxy
 __device__ __forceinline__ void tensormap_acquire(const CUtensorMap *map)
@@ -150,6 +182,9 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) salt_fold_kernel(const __grid
     __shared__ uint64_t full_bar[FOLD_STAGES], empty_bar[FOLD_STAGES];
     __shared__ uint64_t afull_bar[2], aempty_bar[2], tfull_bar[FOLD_NACC], tempty_bar[FOLD_NACC];
     __shared__ uint32_t tmem_slot;
+    // per stage, where its tile goes back to: written by the producer before the stage is full
+    __shared__ const CUtensorMap *st_map[FOLD_STAGES];
+    __shared__ int st_x[FOLD_STAGES], st_y[FOLD_STAGES];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool table = p.mats != nullptr;
@@ -194,29 +229,32 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) salt_fold_kernel(const __grid
     if (warp == 0) {
         // ---------------------------------------------------------- TMA loads
         if (lane == 0) {
-            int n_issued = 0, mat = fold_find(M, nm, i0), mat_seen = -1;
+            int n_issued = 0;
+            FoldCursor cur;
+            cur.start(M, nm, i0);
+            const FoldMat *seen = nullptr;
             for (int j = 0; j < n_my && ok_all; ++j) {
                 const int s = j % FOLD_STAGES;
                 if (j >= FOLD_STAGES && !mbar_wait(smem_u32(&empty_bar[s]), (uint32_t)(j / FOLD_STAGES - 1) & 1u)) {
                     ok_all = false;
                     break;
                 }
-                const int64_t it = i0 + j;
-                fold_advance(M, nm, it, mat);
-                const FoldMat &F = M[mat];
-                if (table && mat != mat_seen) {
+                const FoldMat &F = *cur.F;
+                if (table && cur.F != seen) {
                     tensormap_acquire(&F.wmap);
                     tensormap_acquire(&F.qmap);
-                    mat_seen = mat;
+                    seen = cur.F;
                 }
-                const int n_ct = (F.Ndim + FOLD_NC - 1) / FOLD_NC;
-                const int64_t loc = it - F.item0;
-                const int m0 = (int)(loc / n_ct) * FOLD_TM, n0 = (int)(loc % n_ct) * FOLD_NC;
+                const int m0 = cur.rt * FOLD_TM, n0 = cur.ct * FOLD_NC;
                 const uint32_t sw = st32 + (uint32_t)s * FOLD_STAGE_BYTES, bar = smem_u32(&full_bar[s]);
+                st_map[s] = &F.wmap;
+                st_x[s] = n0;
+                st_y[s] = m0;
                 mbar_expect_tx(bar, (uint32_t)FOLD_W_BYTES + (uint32_t)((F.rc + 15) & ~15) * 128u);
                 tma_load_2d(sw, &F.wmap, n0, m0, bar);
                 tma_load_2d(sw + FOLD_W_BYTES, &F.qmap, n0, 0, bar);
                 n_issued = j + 1;
+                if (j + 1 < n_my) cur.step();
             }
             // every copy issued has landed before the CTA may exit
             for (int j = n_issued - FOLD_STAGES > 0 ? n_issued - FOLD_STAGES : 0; j < n_issued; ++j)
@@ -224,53 +262,47 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) salt_fold_kernel(const __grid
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMAs
-        if (lane == 0) {
-            const uint32_t idesc = idesc_bf16_f32_bmn(FOLD_TM, FOLD_NC);
-            int mat = fold_find(M, nm, i0), key_mat = -1, key_rt = -1, n_tiles = 0, abuf = 0;
-            for (int j = 0; j < n_my && ok_all; ++j) {
-                const int64_t it = i0 + j;
-                fold_advance(M, nm, it, mat);
-                const FoldMat &F = M[mat];
-                const int n_ct = (F.Ndim + FOLD_NC - 1) / FOLD_NC;
-                const int rt = (int)((it - F.item0) / n_ct);
-                if (mat != key_mat || rt != key_rt) {  // a new (weight, row tile): its A tile
-                    abuf = n_tiles & 1;
-                    if (!mbar_wait(smem_u32(&afull_bar[abuf]), (uint32_t)(n_tiles >> 1) & 1u)) { ok_all = false; break; }
-                    ++n_tiles;
-                    key_mat = mat;
-                    key_rt = rt;
-                }
-                const int s = j % FOLD_STAGES, acc = j % FOLD_NACC;
-                if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(j / FOLD_STAGES) & 1u)) { ok_all = false; break; }
-                if (j >= FOLD_NACC && !mbar_wait(smem_u32(&tempty_bar[acc]), (uint32_t)(j / FOLD_NACC - 1) & 1u)) {
-                    ok_all = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t a = a32 + (uint32_t)abuf * FOLD_A_BYTES;
-                const uint32_t q = st32 + (uint32_t)s * FOLD_STAGE_BYTES + FOLD_W_BYTES;
-                const int kpad = (F.rc + 15) & ~15;
+        const uint32_t idesc = idesc_bf16_f32_bmn(FOLD_TM, FOLD_NC);
+        int n_tiles = 0, abuf = 0;
+        bool fresh = true;  // a new (weight, row tile): its A tile
+        FoldCursor cur;
+        cur.start(M, nm, i0);
+        for (int j = 0; j < n_my && ok_all; ++j) {
+            if (fresh) {
+                abuf = n_tiles & 1;
+                if (!mbar_wait(smem_u32(&afull_bar[abuf]), (uint32_t)(n_tiles >> 1) & 1u)) ok_all = false;
+                ++n_tiles;
+            }
+            const int s = j % FOLD_STAGES, acc = j % FOLD_NACC;
+            if (!mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(j / FOLD_STAGES) & 1u)) ok_all = false;
+            if (j >= FOLD_NACC && !mbar_wait(smem_u32(&tempty_bar[acc]), (uint32_t)(j / FOLD_NACC - 1) & 1u)) ok_all = false;
+            ok_all = __all_sync(0xffffffffu, ok_all);
+            if (!ok_all) break;
+            tc_fence_after();
+            const uint32_t a = a32 + (uint32_t)abuf * FOLD_A_BYTES;
+            const uint32_t q = st32 + (uint32_t)s * FOLD_STAGE_BYTES + FOLD_W_BYTES;
+            const int kpad = (cur.F->rc + 15) & ~15;
+            fresh = cur.ends_tile();
+            if (elect_one()) {
                 for (int kk = 0; kk < kpad / 16; ++kk)
                     umma_bf16(tmem + (uint32_t)acc * FOLD_NC, sdesc_kmajor_sw128(a + kk * 32),
                               sdesc_mnmajor_sw128(q + kk * 2048), idesc, kk > 0 ? 1u : 0u);
                 umma_commit(smem_u32(&tfull_bar[acc]));
                 // the A tile is free once the last MMA of its row tile has completed
-                const bool last_of_tile = j + 1 == n_my ||
-                                          (mat + 1 < nm && it + 1 >= M[mat + 1].item0) ||
-                                          (int)((it + 1 - F.item0) / n_ct) != rt;
-                if (last_of_tile) umma_commit(smem_u32(&aempty_bar[abuf]));
+                if (fresh || j + 1 == n_my) umma_commit(smem_u32(&aempty_bar[abuf]));
             }
+            __syncwarp();
+            if (j + 1 < n_my) cur.step();
         }
     } else if (warp == 2) {
         // ---------------------------------------------------------- P^T tiles
         // the CTA's (weight, row tile) pairs in item order
         int64_t it = i0;
-        int mat = fold_find(M, nm, i0);
+        FoldCursor cur;
+        cur.start(M, nm, i0);
         for (int t = 0; it < i1 && ok_all; ++t) {
-            fold_advance(M, nm, it, mat);
-            const FoldMat &F = M[mat];
-            const int n_ct = (F.Ndim + FOLD_NC - 1) / FOLD_NC;
-            const int rt = (int)((it - F.item0) / n_ct);
+            const FoldMat &F = *cur.F;
+            const int n_ct = cur.n_ct, rt = cur.rt;
             const int Mdim = F.Mdim, rc = F.rc, kb_n = ((rc + 15) & ~15) / 8;
             const uint16_t *P = F.P;
             const int b = t & 1;
@@ -307,19 +339,20 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) salt_fold_kernel(const __grid
             fence_async_smem();
             mbar_arrive_release(smem_u32(&afull_bar[b]));
             // the next row tile's first item
-            const int64_t nxt = F.item0 + (int64_t)(rt + 1) * n_ct;
-            it = nxt;
+            it = F.item0 + (int64_t)(rt + 1) * n_ct;
+            cur.ct = n_ct - 1;
+            if (it < i1) cur.step();
         }
     } else {
         // ---------------------------------------------------------- epilogue
-        const int et = tid - 32 * FOLD_EPI_WARP0;
+        const int grp = (warp - FOLD_EPI_WARP0) >> 2, et = tid - 32 * FOLD_EPI_WARP0 - grp * FOLD_EPI_THREADS;
         const int q = warp & 3, r = q * 32 + lane;  // TMEM lane quarter of this warp
         const float scale = p.scale;
-        int mat = fold_find(M, nm, i0), mat_seen = -1;
-        for (int j = 0; j < n_my; ++j) {
+        const CUtensorMap *seen = nullptr;
+        for (int j = grp; j < n_my; j += FOLD_EPI_GROUPS) {
             const int s = j % FOLD_STAGES, acc = j % FOLD_NACC;
-            // the four warps decide together whether to go on, so none is
-            // left at the barrier after another gave up
+            // the group's four warps decide together whether to go on, so none
+            // is left at the barrier after another gave up
             bool ok = mbar_wait(smem_u32(&tfull_bar[acc]), (uint32_t)(j / FOLD_NACC) & 1u) &&
                       mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(j / FOLD_STAGES) & 1u);
             ok = __all_sync(0xffffffffu, ok);
@@ -346,26 +379,21 @@ __global__ void __launch_bounds__(FOLD_THREADS, 1) salt_fold_kernel(const __grid
                 }
                 fence_async_smem();
             }
-            if (!named_sync_and(FOLD_BAR_EPI, FOLD_EPI_THREADS, ok)) {
+            if (!named_sync_and(FOLD_BAR_EPI + grp, FOLD_EPI_THREADS, ok)) {
                 ok_all = false;
                 break;
             }
             if (et == 0) {
-                const int64_t it = i0 + j;
-                fold_advance(M, nm, it, mat);
-                const FoldMat &F = M[mat];
-                if (table && mat != mat_seen) {
-                    tensormap_acquire(&F.wmap);
-                    mat_seen = mat;
+                const CUtensorMap *map = st_map[s];
+                if (table && map != seen) {
+                    tensormap_acquire(map);
+                    seen = map;
                 }
-                const int n_ct = (F.Ndim + FOLD_NC - 1) / FOLD_NC;
-                const int64_t loc = it - F.item0;
-                tma_store_2d(&F.wmap, st32 + (uint32_t)s * FOLD_STAGE_BYTES, (int)(loc % n_ct) * FOLD_NC,
-                             (int)(loc / n_ct) * FOLD_TM);
+                tma_store_2d(map, st32 + (uint32_t)s * FOLD_STAGE_BYTES, st_x[s], st_y[s]);
                 bulk_commit();
-                // the previous item's store has read its stage: hand it back
+                // the group's previous store has read its stage: hand it back
                 bulk_wait_read<1>();
-                if (j >= 1) mbar_arrive_release(smem_u32(&empty_bar[(j - 1) % FOLD_STAGES]));
+                if (j >= FOLD_EPI_GROUPS) mbar_arrive_release(smem_u32(&empty_bar[(j - FOLD_EPI_GROUPS) % FOLD_STAGES]));
             }
         }
         if (et == 0) bulk_wait_all();
