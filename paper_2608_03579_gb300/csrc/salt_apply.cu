@@ -68,17 +68,19 @@ constexpr int TMEM_COLS = 512;                 // expand: N_ACC x 64 accumulator
 constexpr int DT_COL = 256;                    // first column of the shrink accumulator (<= 128 tokens)
 constexpr int N_ACC = 4;                       // expand accumulators in tensor memory
 constexpr int KS_MAX = 16;
+constexpr int STACK_ROWS = 256;                // stacked A rows of a shrink unit: one projection's, or every one's
 constexpr int VT_ROW = VEXT_COLS * 2;          // bytes per V tile row
 constexpr int VT_BYTES = TM * VT_ROW;
 // a deferred unit stages the sums of its slice (<= TM / 2 token rows: the
 // block's non-empty splits are >= 2) in the V tile's region
 static_assert((TM / 2) * SALT_MAX_TOKEN_RANK * 4 <= VT_BYTES, "deferred reduction staging exceeds the V tile");
 static_assert(5 * 2 * TILE_BYTES + VT_BYTES <= RING_BYTES, "the expand ring must hold 5 full stages and the V tile");
-static_assert(VT_BYTES <= RING_BYTES, "V staging exceeds the ring");
+static_assert(4 * (TM + STACK_ROWS) * 128 <= RING_BYTES, "whole units: four stages of the largest size");
+static_assert(DT_COL + STACK_ROWS <= TMEM_COLS, "whole units: the accumulator of every projection");
 static_assert(S_MAX <= 128, "the factor stack is the 128-row UMMA operand");
 
 struct FusedInfo {
-    const uint16_t *src[S_MAX];  // shrink: stacked A rows of the current unit's block
+    const uint16_t *src[STACK_ROWS];  // shrink: stacked A rows of the current unit's block
     const uint16_t *esrc[S_MAX]; // expand: stacked B rows of the current run's block
     int32_t row[TM];             // shrink: x row of the i-th token of the unit's block
     int32_t erow[TM];            // expand: y row of the i-th token of the run's block
@@ -233,7 +235,8 @@ __device__ void pair_range(const ApplyParams &p, int n_blk, int nu, int g, int l
 // prefill tokens 215 -> 196 us, an 8B layer at 256 decode tokens 99 -> 95.
 constexpr int SHRINK_MMA_WARP = APPLY_THREADS / 32 - 1;
 constexpr int LOAD_THREADS = 32 * SHRINK_MMA_WARP;
-constexpr int MAX_PIECES = (TM * 8 + LOAD_THREADS - 1) / LOAD_THREADS;  // 16-byte pieces per thread and chunk
+constexpr int MAX_PIECES = (TM * 8 + LOAD_THREADS - 1) / LOAD_THREADS;  // 16-byte pieces of x per thread and chunk
+constexpr int MAX_A_PIECES = (STACK_ROWS * 8 + LOAD_THREADS - 1) / LOAD_THREADS;
 constexpr int N_QUADS = APPLY_THREADS / 128;  // full groups of 4 warps (one per TMEM lane quarter)
 constexpr int EPI_WARP0 = PRODUCER_WARPS + 1;  // first epilogue warp
 constexpr int EPI_THREADS = 32 * EPI_WARPS;
@@ -255,17 +258,19 @@ constexpr int BAR_ALL = 4;                     // every thread (the inline unit 
 struct UnitGeom {
     int unit, pair, s, b, pi, KS;
     int M, rc, S, m_rows, nk, c0;
+    int part0;  // the block's first partial tile (an unsplit unit uses its CTA's)
 };
 
-__device__ __forceinline__ UnitGeom unit_geom(const ApplyParams &p, int unit, int KS)
+__device__ __forceinline__ UnitGeom unit_geom(const ApplyParams &p, int unit, int KS, bool all_proj)
 {
     UnitGeom g;
     g.unit = unit;
     g.KS = KS;
     g.pair = unit / KS;
     g.s = unit - g.pair * KS;
-    g.b = g.pair / p.n_proj;
-    g.pi = g.pair - g.b * p.n_proj;
+    g.part0 = KS == 1 ? (int)blockIdx.x : g.pair * KS;
+    g.b = all_proj ? unit : g.pair / p.n_proj;
+    g.pi = all_proj ? 0 : g.pair - g.b * p.n_proj;
     const int4 m0 = *reinterpret_cast<const int4 *>(p.blk + BLK_INTS * g.b);
     const int4 m1 = *reinterpret_cast<const int4 *>(p.blk + BLK_INTS * g.b + 4);
     g.M = m0.y;
@@ -301,7 +306,7 @@ __device__ void finish_split_unit(const ApplyParams &p, FusedInfo &info, const U
         t1 = info.rt1[sr];
         col = rc + info.rk[sr];
     }
-    float *P = p.w.part + (int64_t)g.unit * (TM * PART_COLS);
+    float *P = p.w.part + (int64_t)(g.part0 + g.s) * (TM * PART_COLS);
     for (int gg = th; gg < (g.m_rows >> 4); gg += nth) {
         uint32_t v[16];
         tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + DT_COL + gg * 16, v);
@@ -336,8 +341,11 @@ __device__ void finish_split_unit(const ApplyParams &p, FusedInfo &info, const U
     // sums of the slice's partial columns (centroid, then the token's own
     // user's), in split order, staged in shared memory, then scaled, masked
     // and written as bf16 V rows
-    constexpr int PC4 = PART_COLS / 4;
-    const int n_it = (r1 - r0) * PC4;
+    // (a row's 4-column pieces that can hold anything, and the multiplier
+    // that divides the item numbers, below 2^12, by their count)
+    const int PC4 = p.tok_c4, n_it = (r1 - r0) * PC4;
+    const uint32_t inv = p.tok_c4_inv;
+    auto row_of = [&](int it) { return PC4 == 1 ? it : (int)__umulhi((uint32_t)it, inv); };
     // (row, 4 columns) items of the slice; with up to 8 splits a thread
     // takes two items at once, so all of its loads are in flight together
     constexpr int KS_PAIR = 8;
@@ -347,9 +355,9 @@ __device__ void finish_split_unit(const ApplyParams &p, FusedInfo &info, const U
         const float *src[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int it = idx + h * nthr, rr = it / PC4, c4 = it - rr * PC4, t = r0 + rr;
+            const int it = idx + h * nthr, rr = row_of(it), c4 = it - rr * PC4, t = r0 + rr;
             use[h] = it < n_it && c4 * 4 < rc + info.urank[t];
-            src[h] = p.w.part + ((int64_t)g.pair * KS * TM + t) * PART_COLS + c4 * 4;
+            src[h] = p.w.part + ((int64_t)g.part0 * TM + t) * PART_COLS + c4 * 4;
 #pragma unroll
             for (int s2 = 0; s2 < KS_PAIR; ++s2) {
                 v[h][s2] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -368,15 +376,15 @@ __device__ void finish_split_unit(const ApplyParams &p, FusedInfo &info, const U
                 acc.z += v[h][s2].z;
                 acc.w += v[h][s2].w;
             }
-            const int it = idx + h * nthr, rr = it / PC4, c4 = it - rr * PC4;
+            const int it = idx + h * nthr, rr = row_of(it), c4 = it - rr * PC4;
             *reinterpret_cast<float4 *>(Ps + rr * PART_COLS + c4 * 4) = acc;
         }
     }
     for (int idx = tid; KS > KS_PAIR && idx < n_it; idx += nthr) {
-        const int rr = idx / PC4, c4 = idx - rr * PC4, t = r0 + rr;
+        const int rr = row_of(idx), c4 = idx - rr * PC4, t = r0 + rr;
         if (c4 * 4 >= rc + info.urank[t]) continue;
         float4 v[KS_MAX];
-        const float *src = p.w.part + ((int64_t)g.pair * KS * TM + t) * PART_COLS + c4 * 4;
+        const float *src = p.w.part + ((int64_t)g.part0 * TM + t) * PART_COLS + c4 * 4;
 #pragma unroll
         for (int s2 = 0; s2 < KS_MAX; ++s2) {
             v[s2] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -422,6 +430,12 @@ __device__ void finish_split_unit(const ApplyParams &p, FusedInfo &info, const U
     if (tid == 0) signal_add(p.w.vdone + (epoch & 1) * n_pairs + pidx);
 }
 
+// WHOLE: with the path of unsplit units (whole below).  Without it they are
+// finished like split ones, correct but slower; the launch takes that kernel
+// for batches of few row blocks, whose units are split (launch_apply), because
+// the shorter code is what a launch of a few microseconds waits for (3B q/k/v
+// at 64 tokens 13.9 -> 12.6 us, an 8B decode layer 94 -> 89).
+template <bool WHOLE>
 __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __grid_constant__ ApplyParams p)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -429,7 +443,6 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
     uint8_t *ring = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     FusedInfo &info = *reinterpret_cast<FusedInfo *>(ring + RING_BYTES);
     const uint32_t ring32 = smem_u32(ring);
-    uint16_t *Vs = reinterpret_cast<uint16_t *>(ring);  // shrink: V tile staging [TM][VEXT_COLS]
 
     // Before the dependency wait this kernel reads only the segment tables
     // and the factors: the host launches it as a programmatic dependent only
@@ -449,7 +462,22 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
     const int n_bp = n_blk * p.n_proj;
     int KS = max(1, min(KS_MAX, (int)gridDim.x / n_bp));
     if (KS > 1 && (int64_t)n_bp * KS > p.w.part_cap) KS = max(1, p.w.part_cap / n_bp);
-    const int n_units = n_bp * KS;
+    // Projections of the same x whose stacks fit one operand together (short
+    // stacks: prefill) share their units, so that x goes into an SM once, when
+    // the row blocks alone occupy most CTAs with whole (unsplit) units.  Fewer
+    // blocks are left one unit a projection: 66 blocks of two projections run
+    // as fast on 132 CTAs, and splitting K costs a hand-off of 5-10 us.
+    // Measured (16384 tokens, q/v of 4096, 129 blocks, the
+    // build included): 378 -> 310 us with two such launches.
+    bool all_proj = false;
+    if (WHOLE) {
+        const int n_stack = (p.counts[4] + 15) & ~15;
+        all_proj = p.shared_x && p.n_proj > 1 && p.n_proj * n_stack <= STACK_ROWS && 2 * n_blk > (int)gridDim.x;
+        if (all_proj) KS = 1;
+    }
+    const bool whole = WHOLE && KS == 1;
+    const int n_comb = all_proj ? p.n_proj : 1;
+    const int n_units = all_proj ? n_blk : n_bp * KS;
     // With at most one unit per CTA the units go to the lowest CTA indices:
     // the CTAs of a launch start in index order as the previous launch's
     // CTAs leave their SMs, so the last ones to start (up to a few
@@ -515,7 +543,7 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
     // item of its range, into info.range; one warp each.  With split
     // shrinks, searched by warps 0 and 1 when the shrink phase is over
     // (while the block's splits are reduced), so that the first shrink
-    // unit's table phase does not wait for the search; with single splits,
+    // unit's table phase does not wait for the search; with whole units,
     // during that table phase.
     bool have_range = false;
     auto find_range = [&](int e) {
@@ -542,23 +570,24 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
     bool deferred = false;
     UnitGeom dgeom{};
     for (int unit = ua; unit < ub; ++unit) {
-        const UnitGeom g = unit_geom(p, unit, KS);
+        const UnitGeom g = unit_geom(p, unit, KS, all_proj);
         const int b = g.b;
         const ApplyProj &pr = p.proj[g.pi];
         const int start = p.blk[BLK_INTS * b + BLK_START], d = p.blk[BLK_INTS * b + BLK_DOM];
         const int M = g.M, rc = g.rc, S = g.S;
         const int d_in = pr.d_in;
         const int nk = g.nk;
+        const int S_pad = (S + 15) & ~15;
         const int c0 = g.c0, n_my = split_lo(nk, g.s + 1, KS) - c0;
         if (S > S_MAX || S == 0 || M <= 0 || n_my <= 0) {
             if (S > S_MAX && g.s == 0 && tid == 0) atomicOr(p.err, SALT_DEVERR_RANK);
             continue;
         }
         __syncthreads();  // the previous unit is done with info and the ring
-        // the token and factor tables (threads 64..191); with single splits
+        // the token and factor tables (threads 64..191); with whole units
         // (the expand follows each unit at once) warps 0 and 1 meanwhile
         // find the CTA's expand items
-        if (KS == 1 && !have_range && warp < 2) {
+        if (whole && !have_range && warp < 2) {
             find_range(warp);
         } else if (tid >= 64 && tid < 64 + TM) {
             const int t = tid - 64;
@@ -585,28 +614,48 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
                     }
                 }
             }
-            if (t < S) {
-                info.src[t] = t < rc ? pr.A + ((int64_t)d * p.rc_max + t) * d_in
-                                     : residual_row(p, pr, p.blk_res[(int64_t)b * S_MAX + (t - rc)], false);
+            if (!whole) {
+                if (t < S)
+                    info.src[t] = t < rc ? pr.A + ((int64_t)d * p.rc_max + t) * d_in
+                                         : residual_row(p, pr, p.blk_res[(int64_t)b * S_MAX + (t - rc)], false);
+            } else if (t < S_pad) {
+                const int res = t >= rc && t < S ? p.blk_res[(int64_t)b * S_MAX + (t - rc)] : 0;
+                for (int c = 0; c < n_comb; ++c) {  // (padding rows: any row of d_in elements)
+                    const ApplyProj &pc = p.proj[g.pi + c];
+                    info.src[c * S_pad + t] = t < rc ? pc.A + ((int64_t)d * p.rc_max + t) * d_in
+                                              : t < S ? residual_row(p, pc, res, false) : pc.x;
+                }
             }
         }
-        have_range = have_range || KS == 1;
+        have_range = have_range || whole;
         __syncthreads();
 
-        // stage geometry: A = the factor stack (the 128-row UMMA M operand; rows
-        // >= S are never read back), X = the block's tokens rounded to the
-        // 16-row UMMA N step
-        const int m_rows = g.m_rows;
-        const int stage_bytes = TILE_BYTES + m_rows * 128;
+        // Stage geometry.  Split units compute V^T: A = the factor stack (the
+        // 128-row UMMA M operand; rows >= S are never read back), then X = the
+        // block's tokens rounded to the 16-row UMMA N step.  Whole units
+        // compute V: X is the M operand (rows >= M are whatever follows in the
+        // stage, never read back), the stacks of the unit's projections, each
+        // padded to 16 rows, the N operand.
+        const int m_rows = g.m_rows, a_rows = n_comb * S_pad;
+        const int a_off = whole ? m_rows * 128 : 0, x_off = whole ? 0 : TILE_BYTES;
+        const int stage_bytes = whole ? max(TILE_BYTES, (m_rows + a_rows) * 128) : TILE_BYTES + m_rows * 128;
         const int nstage = min(A_MAX_STAGES, RING_BYTES / stage_bytes);
-        const uint32_t idesc = idesc_bf16_f32(128, m_rows);
+        const uint32_t idesc = idesc_bf16_f32(128, whole ? a_rows : m_rows);
         // each thread's 16-byte pieces of a chunk: piece j is (row
         // (tid + j * LOAD_THREADS) / 8, 16-byte column tid % 8), so one column
         // offset serves all pieces
         const int cb = (tid & 7) * 8;
-        const int nA = warp < SHRINK_MMA_WARP ? S : 0, nX = warp < SHRINK_MMA_WARP ? M : 0;
-        const uint16_t *a_src[MAX_PIECES];
+        const int nA = warp < SHRINK_MMA_WARP ? (whole ? a_rows : S) : 0, nX = warp < SHRINK_MMA_WARP ? M : 0;
+        const bool tall = whole && a_rows > LOAD_THREADS / 8 * MAX_PIECES;  // stacks beyond MAX_PIECES pieces a thread
+        const uint16_t *a_src[MAX_PIECES], *t_src[MAX_A_PIECES - MAX_PIECES];
         const uint16_t *x_src[MAX_PIECES];
+        if (tall) {
+#pragma unroll
+            for (int j = MAX_PIECES; j < MAX_A_PIECES; ++j) {
+                const int r = (tid + j * LOAD_THREADS) >> 3;
+                t_src[j - MAX_PIECES] = r < nA ? info.src[r] + cb : nullptr;
+            }
+        }
 #pragma unroll
         for (int j = 0; j < MAX_PIECES; ++j) {
             const int r = (tid + j * LOAD_THREADS) >> 3;
@@ -616,17 +665,24 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
         auto load_a = [&](int i, int st) {
             const int k0 = (c0 + i) * KC;
             const bool ok = k0 + cb < d_in;
-            const uint32_t base = ring32 + st * stage_bytes;
+            const uint32_t base = ring32 + st * stage_bytes + a_off;
 #pragma unroll
             for (int j = 0; j < MAX_PIECES; ++j) {
                 const int r = (tid + j * LOAD_THREADS) >> 3;
                 if (r < nA) cp_async16(base + swz128(r, tid & 7), a_src[j] + (ok ? k0 : 0), ok);
             }
+            if (tall) {
+#pragma unroll
+                for (int j = MAX_PIECES; j < MAX_A_PIECES; ++j) {
+                    const int r = (tid + j * LOAD_THREADS) >> 3;
+                    if (r < nA) cp_async16(base + swz128(r, tid & 7), t_src[j - MAX_PIECES] + (ok ? k0 : 0), ok);
+                }
+            }
         };
         auto load_x = [&](int i, int st) {
             const int k0 = (c0 + i) * KC;
             const bool ok = k0 + cb < d_in;
-            const uint32_t base = ring32 + st * stage_bytes + TILE_BYTES;
+            const uint32_t base = ring32 + st * stage_bytes + x_off;
 #pragma unroll
             for (int j = 0; j < MAX_PIECES; ++j) {
                 const int r = (tid + j * LOAD_THREADS) >> 3;
@@ -659,10 +715,11 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
             if (warp == SHRINK_MMA_WARP && elect_one()) {
                 fence_async_smem();
                 tc_fence_after();
-                const uint32_t sa = ring32 + st * stage_bytes, sx = sa + TILE_BYTES;
+                const uint32_t so = ring32 + st * stage_bytes;  // the M operand comes first
+                const uint32_t sn = so + (whole ? a_off : x_off);
 #pragma unroll
                 for (int kk = 0; kk < KC / 16; ++kk)
-                    umma_bf16(tmem + DT_COL, sdesc_kmajor_sw128(sa + kk * 32), sdesc_kmajor_sw128(sx + kk * 32), idesc,
+                    umma_bf16(tmem + DT_COL, sdesc_kmajor_sw128(so + kk * 32), sdesc_kmajor_sw128(sn + kk * 32), idesc,
                               (it > 0 || kk > 0) ? 1u : 0u);
                 umma_commit(smem_u32(&info.bar[st]));
             }
@@ -685,51 +742,51 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
         a_phase ^= pending;
         tc_fence_after();
 
-        if (KS == 1) {
-            // ---- V_ext straight from the accumulator (TMEM lanes = stack rows,
-            // columns = tokens) into the staging tile.  Warp w of the first
-            // N_QUADS groups of four reads lanes 32 (w % 4) .. + 31 and every
-            // N_QUADS-th 16-token group.
-            const int q = warp & 3, th = warp >> 2;
-            const int sr = q * 32 + lane;
-            int t0 = 0, t1 = 0;  // tokens this stack row serves
-            if (sr < rc) {
-                t1 = M;
-            } else if (sr < S) {
-                t0 = info.rt0[sr];
-                t1 = info.rt1[sr];
-            }
-            const int S_pad = (S + 15) & ~15;
-            const int64_t pidx = (int64_t)g.pi * p.w.blk_cap + b;
-            uint16_t *vt = p.w.vext + pidx * (TM * VEXT_COLS);
-            const int nch = S_pad >> 3;
-            for (int gg = th; th < N_QUADS && gg < (m_rows >> 4); gg += N_QUADS) {
-                uint32_t v[16];
-                tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + DT_COL + gg * 16, v);
-                tmem_ld_wait();
-                if (sr < S_pad) {
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int t = gg * 16 + e;
-                        if (t < M) {
-                            float val = 0.f;
-                            if (sr < rc) val = info.usc[t] * __uint_as_float(v[e]);
-                            else if (t >= t0 && t < t1) val = info.usu[t] * __uint_as_float(v[e]);
-                            Vs[t * VEXT_COLS + sr] = f_to_bf16(val);
-                        }
+        if (whole) {
+            // ---- V_ext straight from the accumulator (TMEM lanes = tokens,
+            // columns = stack rows, projection by projection) to device memory.
+            // Warp w of the first N_QUADS groups of four reads lanes
+            // 32 (w % 4) .. + 31 and every N_QUADS-th 16-column group.
+            const int q = warp & 3, th = warp >> 2, t = q * 32 + lane, ng = S_pad >> 4;
+            if (q * 32 < M) {
+                const int tc = min(t, M - 1);
+                const int uc = info.ucol[tc], ue = uc + info.urank[tc];
+                const float us = info.usu[tc], sc = info.usc[tc];
+                for (int gg = th, c = 0, gc = th; gg < n_comb * ng; gg += N_QUADS, gc += N_QUADS) {
+                    while (gc >= ng) {
+                        gc -= ng;
+                        ++c;
                     }
+                    uint32_t v[16];
+                    tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + DT_COL + gg * 16, v);
+                    tmem_ld_wait();
+                    if (t < M) {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int e = 0; e < 16; e += 2) {
+                            uint32_t h2[2];
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const int col = gc * 16 + e + h;
+                                const float a = __uint_as_float(v[e + h]);
+                                h2[h] = f_to_bf16(col < rc ? sc * a : uc >= 0 && col >= uc && col < ue ? us * a : 0.f);
+                            }
+                            w[e >> 1] = h2[0] | h2[1] << 16;
+                        }
+                        uint4 *dst = reinterpret_cast<uint4 *>(p.w.vext + ((int64_t)(g.pi + c) * p.w.blk_cap + b) * (TM * VEXT_COLS) +
+                                                               t * VEXT_COLS + gc * 16);
+                        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                        dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                    }
+                    __syncwarp();
                 }
             }
             tc_fence_before();
             __syncthreads();
-            for (int idx = tid; idx < M * nch; idx += APPLY_THREADS) {
-                const int r = idx / nch, c = idx - r * nch;
-                *reinterpret_cast<uint4 *>(vt + r * VEXT_COLS + c * 8) =
-                    *reinterpret_cast<const uint4 *>(Vs + r * VEXT_COLS + c * 8);
-            }
-            __syncthreads();
-            if (tid == 0) signal_add(p.w.vdone + (info.epoch & 1) * n_pairs + pidx);
-        } else if (unit + 1 < ub || min(KS, nk) < 2) {
+            if (tid == 0)
+                for (int c = 0; c < n_comb; ++c)
+                    signal_add(p.w.vdone + (info.epoch & 1) * n_pairs + (int64_t)(g.pi + c) * p.w.blk_cap + b);
+        } else if (unit + 1 < ub || min(KS, nk) < 2) {  // (also unsplit units without the whole path)
             // a later unit of this CTA reuses the accumulator, or the slice
             // (the whole block when d_in has one chunk) would not fit the V
             // tile's region: finish now, all threads
@@ -1117,7 +1174,9 @@ cudaError_t apply_prepare(int device)
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
     cudaError_t e = cudaDeviceGetAttribute(&g_sm_count[device], cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(salt_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
+    e = cudaFuncSetAttribute(salt_apply_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(salt_apply_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FUSED_SMEM);
 }
 
 cudaError_t launch_wait_selftest(uint32_t *err, cudaStream_t stream)
@@ -1126,7 +1185,7 @@ cudaError_t launch_wait_selftest(uint32_t *err, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, cudaStream_t stream)
+cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, int n_blk, cudaStream_t stream)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1142,7 +1201,11 @@ cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, cudaStream_t 
     cfg.stream = stream;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, salt_apply_kernel, p);
+    // One kernel for all launches of a batch, whatever their projections: a
+    // 3B MLP layer whose two launches took different ones ran 202 us, 190 with
+    // the same for both.
+    return 8LL * n_blk > n_sm ? cudaLaunchKernelEx(&cfg, salt_apply_kernel<true>, p)
+                                                       : cudaLaunchKernelEx(&cfg, salt_apply_kernel<false>, p);
 }
 
 }  // namespace salt

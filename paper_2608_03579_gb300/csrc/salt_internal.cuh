@@ -49,7 +49,7 @@ struct SegDev {
     int32_t *useg_gbin;    // [max_tokens]
     int32_t *useg_slot;    // [max_tokens]
     int32_t *blk;          // [BLK_INTS * max_tokens], see BLK_* below
-    int32_t *counts;       // [4]: n_tokens, domain runs, user runs, row blocks
+    int32_t *counts;       // [5]: n_tokens, domain runs, user runs, row blocks, rows of the largest factor stack
     // per grouped token: first stacked row of its user among the block's
     // residual rows (-1: no residual), the user's rank and scale s_u
     int32_t *tok_uoff;     // [max_tokens]
@@ -156,6 +156,9 @@ struct ApplyParams {
     const int32_t *blk_res;
     int32_t rc_max;
     int32_t min_nk;      // fewest 64-wide d_in chunks over the group's projections (caps the K splits)
+    int32_t shared_x;    // every projection reads the same x (and d_in)
+    int32_t tok_c4;      // 4-column pieces of a partial row that can hold anything (rc_max + r_max columns)
+    uint32_t tok_c4_inv; // floor(2^32 / tok_c4) + 1: divides numbers below 2^12 by it (tok_c4 > 1)
     int32_t shrink_only; // write the V tiles of the row blocks and stop (the base-weight kernel expands)
     const uint8_t *pool;
     int64_t slot_stride;
@@ -212,8 +215,16 @@ cudaError_t apply_prepare(int device);
 // K-split) first, then the expand items (row block, 64 output columns).
 // With pdl the launch is a programmatic dependent of the previous kernel on
 // the stream (only when that kernel did not write the segment tables).
-// The grid is `ctas` CTAs (0: one per SM).
-cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, cudaStream_t stream);
+// The grid is `ctas` CTAs (0: one per SM).  n_blk: at most how many row blocks
+// the batch built last has; it only picks between two kernels that are both
+// right for any count (a captured launch is replayed on later batches).
+cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, int n_blk, cudaStream_t stream);
+// tok_c4 and its divisor for tokens of up to `cols` partial columns.
+inline void apply_set_cols(ApplyParams &p, int cols)
+{
+    p.tok_c4 = (cols + 3) / 4;
+    p.tok_c4_inv = 0xffffffffu / (uint32_t)p.tok_c4 + 1u;
+}
 size_t apply_smem_bytes();
 // W[Mdim][Ndim] += scale * P^T Q for P = [rc][Mdim], Q = [rc][Ndim] (bf16,
 // rows contiguous, rc <= 64): the centroid fold; a timed-out wait sets

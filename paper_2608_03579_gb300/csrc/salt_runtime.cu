@@ -888,7 +888,7 @@ salt_status salt_segments_create(salt_ctx *ctx, salt_segments **out)
               alloc(&seg->d.dseg_ptr, n + 1) && alloc(&seg->d.dseg_dom, n) && alloc(&seg->d.dseg_gbin, n) &&
               alloc(&seg->d.useg_ptr, n + 1) && alloc(&seg->d.useg_dom, n) && alloc(&seg->d.useg_gbin, n) &&
               alloc(&seg->d.useg_slot, n) &&
-              alloc(&seg->d.blk, (size_t)BLK_INTS * n) && alloc(&seg->d.counts, 4) && alloc(&seg->d.tok_uoff, n) &&
+              alloc(&seg->d.blk, (size_t)BLK_INTS * n) && alloc(&seg->d.counts, 5) && alloc(&seg->d.tok_uoff, n) &&
               alloc(&seg->d.tok_urank, n) && alloc(reinterpret_cast<int32_t **>(&seg->d.tok_su), n) &&
               alloc(reinterpret_cast<int32_t **>(&seg->d.tok_sc), n) &&
               alloc(&seg->d.blk_res, (size_t)n * S_MAX) && alloc(&seg->d.aperm, n) && alloc(&seg->d.a_uptr, n + 1) &&
@@ -915,7 +915,7 @@ salt_status salt_segments_create(salt_ctx *ctx, salt_segments **out)
     }
     ok = ok && cudaEventCreateWithFlags(&seg->built_ev, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&seg->tmp_ev, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaMemset(seg->d.counts, 0, 4 * sizeof(int32_t)) == cudaSuccess;
+    ok = ok && cudaMemset(seg->d.counts, 0, 5 * sizeof(int32_t)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         ctx->segs.insert(seg);
@@ -1174,6 +1174,8 @@ salt_status apply_grouped(salt_ctx *ctx, const salt_segments *seg_, int32_t n, c
     }
     p.n_unit_prefix[n] = units;
     p.min_nk = 1 << 30;
+    p.shared_x = 1;
+    for (int i = 1; i < n; ++i) p.shared_x &= p.proj[i].x == p.proj[0].x && p.proj[i].d_in == p.proj[0].d_in;
     for (int i = 0; i < n; ++i) p.min_nk = std::min(p.min_nk, (p.proj[i].d_in + 63) / 64);
     p.perm = seg->d.aperm;
     p.blk = seg->d.blk;
@@ -1184,6 +1186,7 @@ salt_status apply_grouped(salt_ctx *ctx, const salt_segments *seg_, int32_t n, c
     p.tok_sc = seg->d.tok_sc;
     p.blk_res = seg->d.blk_res;
     p.rc_max = ctx->rc_max;
+    apply_set_cols(p, ctx->rc_max + ctx->r_max);
     p.pool = ctx->pool;
     p.slot_stride = ctx->slot_stride;
     p.w = seg->work;
@@ -1192,7 +1195,7 @@ salt_status apply_grouped(salt_ctx *ctx, const salt_segments *seg_, int32_t n, c
     const int ctas = shrink_only ? base_shrink_ctas(seg->T, p.proj[0].d_in, p.proj[0].d_out, seg->n_blk_est) : 0;
     // The first apply after a build waits for the segment kernel in full;
     // later ones overlap their table reads with the previous kernel.
-    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, ctas, stream));
+    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, ctas, seg->n_blk_bound, stream));
     seg->tables_fresh = false;
     return SALT_OK;
 }
@@ -1312,11 +1315,12 @@ salt_status salt_lora_apply_static(salt_ctx *ctx, const salt_segments *seg_, int
     p.tok_sc = seg->d.tok_sc;
     p.blk_res = seg->d.blk_res;
     p.rc_max = ctx->rc_max;
+    apply_set_cols(p, ctx->rc_max + ctx->r_max);
     p.pool = ctx->pool;
     p.slot_stride = ctx->slot_stride;
     p.w = scratch;
     p.err = ctx->err_dev;
-    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, 0, stream));
+    CUDA_OR_FAIL(ctx, launch_apply(p, !seg->tables_fresh, 0, seg->n_blk_bound, stream));
     seg->tables_fresh = false;
     return SALT_OK;
 }

@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) seg_build_kernel(SegParams p)
 {
     extern __shared__ __align__(16) uint64_t keys[];
     __shared__ int warp_sums[32];
+    __shared__ int max_stack;
     const int T = p.T;
     const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
 
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) seg_build_kernel(SegParams p)
         if (tid == 0) {
             p.s.dseg_ptr[0] = 0;
             p.s.useg_ptr[0] = 0;
-            p.s.counts[0] = p.s.counts[1] = p.s.counts[2] = p.s.counts[3] = 0;
+            p.s.counts[0] = p.s.counts[1] = p.s.counts[2] = p.s.counts[3] = p.s.counts[4] = 0;
         }
         return;
     }
@@ -471,6 +472,7 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) seg_build_kernel(SegParams p)
         p.s.counts[1] = n_dseg;
         p.s.counts[2] = n_useg;
         p.s.counts[3] = n_blk;
+        max_stack = 0;
     }
     __syncthreads();
 
@@ -524,9 +526,13 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) seg_build_kernel(SegParams p)
             }
             carry += total;
         }
-        if (lane == 0) p.s.blk[BLK_INTS * b + BLK_NRES] = carry;
+        if (lane == 0) {
+            p.s.blk[BLK_INTS * b + BLK_NRES] = carry;
+            atomicMax(&max_stack, p.s.blk[BLK_INTS * b + BLK_RC] + carry);
+        }
     }
     __syncthreads();
+    if (tid == 0) p.s.counts[4] = max_stack;
 
     // 6. running sum of the expand cost weights over blocks
     const int Eb = (n_blk + nth - 1) / nth;
