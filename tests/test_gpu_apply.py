@@ -220,3 +220,77 @@ def test_apply_argument_errors(salt_lib, wl):
         with pytest.raises(salt.SaltError) as e:
             salt.salt_lora_apply_grouped(r.ctx, r.seg, [0] * 9, [x] * 9, [y] * 9)
         assert e.value.name == "SALT_ERR_INVALID_ARG"
+
+
+def _many_blocks(wl, T, rc, d_in, d_outs):
+    """A batch of over 76 row blocks (more than half of the SMs), its users in
+    random order, some tokens without a term."""
+    n_users = 40
+    u = (wl.uniform(41, 1, T) * n_users).astype(np.int32) % n_users
+    dom, slot = (u % 2).astype(np.int32), u.copy()
+    none = wl.uniform(41, 2, T) < 0.05
+    dom[none], slot[none] = -1, -1
+    return wl.Workload("many_blocks", 41, [("p", d_in, d) for d in d_outs], 2, [rc, max(1, rc - 3)], n_users,
+                       [1, 2] * (n_users // 2), dom_ids=dom, slot_ids=slot)
+
+
+def _check_shared_x(oracle_mod, w, ys, what):
+    from paper_2608_03579_gb300.runner import bf16_bits
+    rows = np.unique(np.concatenate([np.arange(0, w.T, 61), [0, 1, 127, 128, w.T - 1]]))
+    for l, y in enumerate(ys):
+        cents, res = oracle_tables(w, l)
+        ref = oracle_mod.apply(w.x(0, rows), w.y_in(l, rows), w.dom_ids[rows], w.slot_ids[rows], cents, res)
+        assert_close(bf16_bits(y)[rows], ref, f"{what}, projection {l}")
+
+
+@pytest.mark.parametrize("rc,d_in,d_outs,share", [
+    (5, 72, (136, 64, 264), True),     # three stacks of 48 rows in one operand, one K chunk and a remainder
+    (64, 520, (136, 72), True),        # two of 96: more rows than a thread's first pieces
+    (64, 136, (64, 136, 72), True),    # three of 96 do not fit: a unit each
+    (5, 136, (136, 64), False),        # another x each: a unit each
+])
+def test_unsplit_units(salt_lib, oracle_mod, wl, rc, d_in, d_outs, share):
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_tensor
+    w = _many_blocks(wl, 11000, rc, d_in, d_outs)
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        r.build()
+        assert len(r.export()["blocks"]) > 76
+        xs, ys = r.alloc_xy(range(len(d_outs)))
+        xs = [xs[0]] * len(xs) if share else [bf16_tensor(w.x(0)) for _ in xs]
+        r.apply(list(range(len(d_outs))), xs, ys)
+        torch.cuda.synchronize()
+        assert r.device_error() == 0
+        assert salt_lib.salt_guard_check(r.ctx, r.seg) == 0
+        _check_shared_x(oracle_mod, w, ys, "unsplit units")
+
+
+def test_captured_launch_replayed_on_a_larger_batch(salt_lib, oracle_mod, wl):
+    """A launch captured on a batch of a few row blocks, replayed after a build
+    of many: its kernel finishes unsplit units too."""
+    from paper_2608_03579_gb300.runner import SaltRunner
+    w = _many_blocks(wl, 11000, 16, 136, (136, 64))
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        xs, ys = r.alloc_xy([0, 1])
+        xs = [xs[0]] * 2
+        keep = [y.clone() for y in ys]
+        s = torch.cuda.Stream()
+        r.build(w.dom_ids[:40], w.slot_ids[:40], stream=s)
+        r.apply([0, 1], xs, ys, stream=s)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            r.apply([0, 1], xs, ys, stream=s)
+        r.build(stream=s)
+        for y, k in zip(ys, keep):
+            y.copy_(k)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(s):
+            g.replay()
+        torch.cuda.synchronize()
+        assert r.device_error() == 0
+        assert salt_lib.salt_guard_check(r.ctx, r.seg) == 0
+        _check_shared_x(oracle_mod, w, ys, "replayed on a larger batch")
