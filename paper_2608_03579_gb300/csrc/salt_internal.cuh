@@ -38,7 +38,7 @@ __host__ __device__ constexpr int blk_weight(int M, int S) { return 2 * M + S + 
 
 // Device arrays of one segments object.
 struct SegDev {
-    int32_t *ids;          // [3 * max_tokens]: domain ids, slot ids, then gamma bins
+    int32_t *ids;          // [3 * max_tokens]: copies of device ids the kernel cannot read in place
     int32_t *perm;         // [max_tokens] token index in grouped order
     int32_t *sorted_slot;  // [max_tokens] validated slot of the i-th grouped token (-1: none)
     int32_t *dseg_ptr;     // [max_tokens + 1] runs of equal (domain, gamma bin)
@@ -114,15 +114,19 @@ constexpr int PART_CAP = 512;  // partial tiles per segments object (20 MiB)
 
 struct SegParams {
     SegDev s;
+    // the ids where they lie: the caller's device arrays, or the pinned host
+    // staging, which the kernel reads over the host link.  Copying the few KB
+    // queued them behind a step's swap on the copy engine: an 8B decode step
+    // with 64 swaps (four layers) took 768 us, 538 read in place.
+    const int32_t *dom_ids, *slot_ids, *gb_ids;
     int32_t T;
-    int32_t max_tokens;
     int32_t n_domains;
     int32_t n_slots;
     int32_t r_max;
     int32_t umax;
     const int32_t *dom_rc;   // [n_domains] pinned rank, 0 = not pinned
     const float *dom_sc;     // [n_domains] centroid scale
-    int32_t has_gbin;        // ids hold gamma bins
+    int32_t has_gbin;        // gb_ids holds gamma bins
     int32_t n_gamma;         // gamma bins of this build
     float gamma[SALT_MAX_GAMMA_BINS];
     const uint8_t *pool;     // slot pool base

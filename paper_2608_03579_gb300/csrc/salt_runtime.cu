@@ -59,7 +59,7 @@ struct salt_ctx {
 struct salt_segments {
     salt_ctx *ctx = nullptr;
     SegDev d{};
-    int32_t *staging[2] = {nullptr, nullptr};  // pinned host [2 * max_tokens]
+    int32_t *staging[2] = {nullptr, nullptr};  // pinned host [3 * max_tokens], read by the segment kernel
     cudaEvent_t staging_ev[2] = {nullptr, nullptr};
     bool staging_used[2] = {false, false};
     int staging_next = 0;
@@ -238,6 +238,18 @@ bool is_device_pointer(const void *p)
         return false;
     }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+}
+
+// Whether a kernel on `device` can read int32s at p in place (a device
+// array may belong to another device, which only copies reach).
+bool readable_in_place(const void *p, int device)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (reinterpret_cast<uintptr_t>(p) & 3) == 0 && a.type == cudaMemoryTypeDevice && a.device == device;
 }
 
 void add_stream(std::vector<cudaStream_t> &v, cudaStream_t s)
@@ -910,7 +922,7 @@ salt_status salt_segments_create(salt_ctx *ctx, salt_segments **out)
          cudaMemset(seg->work.base_ctr, 0, BASE_CTRS * sizeof(uint32_t)) == cudaSuccess &&
          apply_encode_vmap(seg->work) == cudaSuccess;
     for (int i = 0; ok && i < 2; ++i) {
-        ok = cudaHostAlloc(&seg->staging[i], 3 * (size_t)n * sizeof(int32_t), cudaHostAllocDefault) == cudaSuccess &&
+        ok = cudaHostAlloc(&seg->staging[i], 3 * (size_t)n * sizeof(int32_t), cudaHostAllocMapped) == cudaSuccess &&
              cudaEventCreateWithFlags(&seg->staging_ev[i], cudaEventDisableTiming) == cudaSuccess;
     }
     ok = ok && cudaEventCreateWithFlags(&seg->built_ev, cudaEventDisableTiming) == cudaSuccess &&
@@ -1019,32 +1031,33 @@ salt_status salt_build_segments_gamma(salt_ctx *ctx, salt_segments *seg, const i
         ctx->slot_waited_seq[s] = ctx->slot_seq[s];
         ctx->slot_waited_stream[s] = stream;
     }
-    if (T > 0) {
-        const int32_t *src[3] = {domain_ids, slot_ids, gamma_bins};
-        const int n_arr = has_gbin ? 3 : 2;
-        if (dev_ids) {
-            for (int a = 0; a < n_arr; ++a)
-                CUDA_OR_FAIL(ctx, cudaMemcpyAsync(seg->d.ids + (size_t)a * ctx->max_tokens, src[a], (size_t)T * 4,
-                                                  cudaMemcpyDeviceToDevice, stream));
-        } else {
-            int k = seg->staging_next;
-            seg->staging_next ^= 1;
-            if (seg->staging_used[k]) CUDA_OR_FAIL(ctx, cudaEventSynchronize(seg->staging_ev[k]));
-            int32_t *h = seg->staging[k];
-            for (int a = 0; a < n_arr; ++a) {
-                std::memcpy(h + (size_t)a * ctx->max_tokens, src[a], (size_t)T * 4);
-                CUDA_OR_FAIL(ctx, cudaMemcpyAsync(seg->d.ids + (size_t)a * ctx->max_tokens,
-                                                  h + (size_t)a * ctx->max_tokens, (size_t)T * 4,
-                                                  cudaMemcpyHostToDevice, stream));
-            }
-            CUDA_OR_FAIL(ctx, cudaEventRecord(seg->staging_ev[k], stream));
-            seg->staging_used[k] = true;
+    // The kernel reads device ids in place where it can (else a copy of them),
+    // host ids from a pinned staging area.
+    const int32_t *ids[3] = {domain_ids, slot_ids, gamma_bins};
+    int k = -1;
+    if (T > 0 && !dev_ids) {
+        k = seg->staging_next;
+        seg->staging_next ^= 1;
+        if (seg->staging_used[k]) CUDA_OR_FAIL(ctx, cudaEventSynchronize(seg->staging_ev[k]));
+        for (int a = 0; a < (has_gbin ? 3 : 2); ++a) {
+            int32_t *h = seg->staging[k] + (size_t)a * ctx->max_tokens;
+            std::memcpy(h, ids[a], (size_t)T * 4);
+            ids[a] = h;
+        }
+    } else if (T > 0) {
+        for (int a = 0; a < (has_gbin ? 3 : 2); ++a) {
+            if (readable_in_place(ids[a], ctx->device)) continue;
+            int32_t *d = seg->d.ids + (size_t)a * ctx->max_tokens;
+            CUDA_OR_FAIL(ctx, cudaMemcpyAsync(d, ids[a], (size_t)T * 4, cudaMemcpyDefault, stream));
+            ids[a] = d;
         }
     }
     SegParams p;
     p.s = seg->d;
+    p.dom_ids = ids[0];
+    p.slot_ids = ids[1];
+    p.gb_ids = ids[2];
     p.T = T;
-    p.max_tokens = ctx->max_tokens;
     p.n_domains = ctx->n_domains;
     p.n_slots = ctx->n_slots;
     p.r_max = ctx->r_max;
@@ -1058,6 +1071,10 @@ salt_status salt_build_segments_gamma(salt_ctx *ctx, salt_segments *seg, const i
     p.slot_stride = ctx->slot_stride;
     p.err = ctx->err_dev;
     CUDA_OR_FAIL(ctx, launch_segments(p, stream));
+    if (k >= 0) {
+        CUDA_OR_FAIL(ctx, cudaEventRecord(seg->staging_ev[k], stream));
+        seg->staging_used[k] = true;
+    }
     CUDA_OR_FAIL(ctx, cudaEventRecord(seg->built_ev, stream));
 
     seg->built = true;

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(SEG_THREADS, 1) seg_build_kernel(SegParams p)
 
     // 1. validate and build keys
     uint32_t errbits = 0;
-    const int32_t *dom_ids = p.s.ids, *slot_ids = p.s.ids + p.max_tokens, *gb_ids = p.s.ids + 2 * p.max_tokens;
+    const int32_t *dom_ids = p.dom_ids, *slot_ids = p.slot_ids, *gb_ids = p.gb_ids;
     for (int i0 = 0; i0 < R; i0 += LOAD_BATCH) {
         int d[LOAD_BATCH], sl[LOAD_BATCH], gb[LOAD_BATCH], rc[LOAD_BATCH], rk[LOAD_BATCH];
         uint64_t magic[LOAD_BATCH];
