@@ -243,6 +243,10 @@ cudaError_t fold_record(void *rec, const uint16_t *P, const uint16_t *Q, uint16_
                         int64_t item0, int64_t *n_items);
 // Every weight of a device table of n records (items in all) in one launch.
 cudaError_t launch_fold_table(const void *table, int n, int64_t items, float scale, uint32_t *err, cudaStream_t stream);
+// n blobs (16-byte aligned, bytes a multiple of 16, readable by the device)
+// from host memory into device memory by one kernel.
+cudaError_t swap_prepare();
+cudaError_t launch_swap(int n, const void *const *src, void *const *dst, const uint64_t *bytes, cudaStream_t stream);
 // salt_align_loss on the current device.
 salt_status align_loss_run(int32_t n, const salt_align_pair *pairs, float eps, float *loss, float *cosine,
                            cudaStream_t stream);

@@ -47,7 +47,17 @@ struct salt_ctx {
     int64_t slot_stride = 0;
     std::vector<int32_t> slot_rank;        // 0 = never loaded
     std::vector<uint64_t> slot_seq;        // loads issued
-    std::vector<cudaEvent_t> slot_ready;
+    std::vector<cudaEvent_t> slot_ready;   // recorded by the slot's own load
+    // Loads made by one launch share an event: slot_batch[s] is its index (-1:
+    // slot_ready[s]); an event is recorded again only once no slot's last load
+    // is its batch.
+    struct BatchEvent {
+        cudaEvent_t ev;
+        int slots;
+    };
+    std::vector<BatchEvent> batch_events;
+    std::vector<int32_t> slot_batch;
+    bool direct_host = false;              // kernels read registered host memory at its host address
     std::vector<uint64_t> slot_waited_seq;
     std::vector<cudaStream_t> slot_waited_stream;
 
@@ -380,9 +390,42 @@ salt_status check_blob(salt_ctx *ctx, int32_t slot, const void *host_blob, int32
     return SALT_OK;
 }
 
+// The batch event of a new load: one that no slot refers to, or a new one.
+cudaError_t take_batch_event(salt_ctx *ctx, int32_t *index)
+{
+    for (size_t i = 0; i < ctx->batch_events.size(); ++i)
+        if (ctx->batch_events[i].slots == 0) {
+            *index = (int32_t)i;
+            return cudaSuccess;
+        }
+    cudaEvent_t ev;
+    const cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) return e;
+    ctx->batch_events.push_back({ev, 0});
+    *index = (int32_t)ctx->batch_events.size() - 1;
+    return cudaSuccess;
+}
+
+// Slot `slot` holds a new load: recorded in batch event `batch`, or (-1) in
+// the slot's own event.
+void slot_loaded(salt_ctx *ctx, int32_t slot, int32_t rank, int32_t batch)
+{
+    if (ctx->slot_batch[slot] >= 0) ctx->batch_events[ctx->slot_batch[slot]].slots -= 1;
+    if (batch >= 0) ctx->batch_events[batch].slots += 1;
+    ctx->slot_batch[slot] = batch;
+    ctx->slot_rank[slot] = rank;
+    ctx->slot_seq[slot] += 1;
+}
+
+// Loads of one launch: at least this many blobs, in library host regions.
+// (A single blob is one copy-engine copy, 6.5 us for 1.31 MB.)
+constexpr int SWAP_LAUNCH_MIN = 4;
+
 // The loads of n checked blobs on `side`: readers first (every segments
-// object that names one of the slots waits for its uses, once), then one
-// copy and one ready event per slot.
+// object that names one of the slots waits for its uses, once), then the
+// blobs by one launch and a ready event of all, or one copy and one ready
+// event per slot.  The launch reads the blobs by the device, so it is taken
+// where all lie in this library's own host regions, on 16-byte boundaries.
 salt_status enqueue_loads(salt_ctx *ctx, int32_t n, const int32_t *slots, const void *const *blobs, const int32_t *ranks,
                           const uint64_t *bytes, cudaStream_t side)
 {
@@ -394,13 +437,30 @@ salt_status enqueue_loads(salt_ctx *ctx, int32_t n, const int32_t *slots, const 
         seg->stale = true;
         CUDA_OR_FAIL(ctx, wait_for_uses(seg, side));
     }
+    bool launch = n >= SWAP_LAUNCH_MIN && ctx->direct_host;
+    for (int32_t i = 0; i < n && launch; ++i)
+        launch = (reinterpret_cast<uintptr_t>(blobs[i]) & 15) == 0 && (bytes[i] & 15) == 0 && in_host_region(blobs[i], bytes[i]);
+    if (launch) {  // (a slot named twice is loaded in order, by copies)
+        std::vector<int32_t> sorted(slots, slots + n);
+        std::sort(sorted.begin(), sorted.end());
+        launch = std::adjacent_find(sorted.begin(), sorted.end()) == sorted.end();
+    }
+    if (launch) {
+        std::vector<void *> dst(n);
+        for (int32_t i = 0; i < n; ++i) dst[i] = ctx->pool + (int64_t)slots[i] * ctx->slot_stride;
+        int32_t batch = -1;
+        CUDA_OR_FAIL(ctx, take_batch_event(ctx, &batch));
+        CUDA_OR_FAIL(ctx, launch_swap(n, blobs, dst.data(), bytes, side));
+        CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->batch_events[batch].ev, side));
+        for (int32_t i = 0; i < n; ++i) slot_loaded(ctx, slots[i], ranks[i], batch);
+        return SALT_OK;
+    }
     for (int32_t i = 0; i < n; ++i) {
         const int32_t slot = slots[i];
         uint8_t *dst = ctx->pool + (int64_t)slot * ctx->slot_stride;
         CUDA_OR_FAIL(ctx, cudaMemcpyAsync(dst, blobs[i], bytes[i], cudaMemcpyHostToDevice, side));
         CUDA_OR_FAIL(ctx, cudaEventRecord(ctx->slot_ready[slot], side));
-        ctx->slot_rank[slot] = ranks[i];
-        ctx->slot_seq[slot] += 1;
+        slot_loaded(ctx, slot, ranks[i], -1);
     }
     return SALT_OK;
 }
@@ -565,12 +625,16 @@ salt_status salt_ctx_create(const salt_config *config, salt_ctx **out)
     ctx->slot_waited_seq.assign(ns, 0);
     ctx->slot_waited_stream.assign(ns, nullptr);
     ctx->slot_ready.assign(ns, nullptr);
+    ctx->slot_batch.assign(ns, -1);
+    int direct = 0;
+    ctx->direct_host =
+        cudaDeviceGetAttribute(&direct, cudaDevAttrCanUseHostPointerForRegisteredMem, ctx->device) == cudaSuccess && direct;
     for (int s = 0; s < ns; ++s)
         if (cudaEventCreateWithFlags(&ctx->slot_ready[s], cudaEventDisableTiming) != cudaSuccess)
             return cleanup_fail(SALT_ERR_CUDA);
     if (cudaMalloc(&ctx->err_dev, sizeof(uint32_t)) != cudaSuccess) return cleanup_fail(SALT_ERR_OOM);
     if (cudaMemset(ctx->err_dev, 0, sizeof(uint32_t)) != cudaSuccess) return cleanup_fail(SALT_ERR_CUDA);
-    if (apply_prepare(ctx->device) != cudaSuccess || base_prepare(ctx->device) != cudaSuccess) {
+    if (apply_prepare(ctx->device) != cudaSuccess || base_prepare(ctx->device) != cudaSuccess || swap_prepare() != cudaSuccess) {
         cudaGetLastError();
         return cleanup_fail(SALT_ERR_CUDA);
     }
@@ -590,6 +654,7 @@ void salt_ctx_destroy(salt_ctx *ctx)
     cudaFree(ctx->dom_sc_dev);
     guarded_free(ctx->pool);
     cudaFree(ctx->err_dev);
+    for (auto &b : ctx->batch_events) cudaEventDestroy(b.ev);
     for (cudaEvent_t e : ctx->slot_ready)
         if (e) cudaEventDestroy(e);
     cudaGetLastError();
@@ -1023,11 +1088,15 @@ salt_status salt_build_segments_gamma(salt_ctx *ctx, salt_segments *seg, const i
     // The device buffers of seg may still be read by earlier uses on other streams.
     CUDA_OR_FAIL(ctx, wait_for_uses(seg, stream));
     // Swaps of the slots this batch reads must land first.
+    int32_t last_batch = -1;
     for (int s = 0; s < ctx->n_slots; ++s) {
         if (!(dev_ids ? true : refs[s])) continue;
         if (ctx->slot_seq[s] == 0) continue;
         if (ctx->slot_waited_seq[s] == ctx->slot_seq[s] && ctx->slot_waited_stream[s] == stream) continue;
-        CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(stream, ctx->slot_ready[s], 0));
+        const int32_t bt = ctx->slot_batch[s];
+        if (bt < 0 || bt != last_batch)  // (a batch's slots follow each other more often than not)
+            CUDA_OR_FAIL(ctx, cudaStreamWaitEvent(stream, bt < 0 ? ctx->slot_ready[s] : ctx->batch_events[bt].ev, 0));
+        if (bt >= 0) last_batch = bt;
         ctx->slot_waited_seq[s] = ctx->slot_seq[s];
         ctx->slot_waited_stream[s] = stream;
     }

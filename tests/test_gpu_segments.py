@@ -144,3 +144,17 @@ def test_device_id_errors_raise_flags(salt_lib, oracle_mod):
         salt.salt_segments_destroy(seg)
     finally:
         salt.salt_ctx_destroy(ctx)
+
+
+def test_segments_device_ids_off_their_alignment(env, oracle_mod, wl):
+    """Device ids the kernel cannot read in place (not on a 4-byte boundary)
+    are copied first."""
+    salt, ctx, seg = env
+    dom, slot = _ids(wl, 777, 9, 513, seed=5)
+    buf = [torch.zeros(4 * 777 + 8, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    for b, ids in zip(buf, (dom, slot)):
+        b[2:2 + 4 * 777] = torch.from_numpy(ids.view(np.uint8).copy()).cuda()
+    torch.cuda.synchronize()
+    salt.salt_build_segments(ctx, seg, buf[0].data_ptr() + 2, buf[1].data_ptr() + 2, n_tokens=777)
+    _check(salt, ctx, seg, oracle_mod, dom, slot, umax=(128 - 16) // 2)
+    assert salt.salt_get_device_error(ctx) == 0

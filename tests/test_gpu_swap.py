@@ -195,3 +195,51 @@ def test_batch_load_between_batches_on_side_stream(salt_lib, oracle_mod, wl):
     assert_close(got1, _oracle(oracle_mod, w, lambda u: 0), "before the batch")
     assert_close(got2, _oracle(oracle_mod, w, lambda u: 0), "after the refused batch")
     assert_close(got3, _oracle(oracle_mod, w, lambda u: 5 if u in (0, 2, 5) else 0), "after the batch")
+
+
+@pytest.mark.parametrize("slots,shift", [
+    ([0, 1, 2, 3, 4, 5], 0),   # one launch
+    ([6, 1, 3, 0, 5], 0),      # the same, slots in no order
+    ([6, 1, 3, 0, 5], 8),      # blobs off the 16-byte boundaries: copies
+    ([2, 1, 3, 2, 5], 0),      # a slot named twice: copies, the last one stays
+])
+def test_batch_load_from_a_host_region(salt_lib, oracle_mod, wl, slots, shift):
+    """Batches the swap kernel takes and ones it must not: ranks 1 and 2, blob
+    sizes that are no multiple of a CTA's piece, loaded twice so that a batch's
+    event is used again."""
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
+    salt = salt_lib
+    T = 48
+    u = (wl.uniform(31, 1, T) * 8).astype(np.int32) % 8
+    w = wl.Workload("swap_region", 31, [("p", 2056, 384), ("q", 4096, 1032)], 2, [16, 16], 8, [1, 2] * 4, dom_ids=u % 2,
+                    slot_ids=u)
+    side, comp = torch.cuda.Stream(), torch.cuda.Stream()
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        step = (r.blob_bytes(2) + 255) // 256 * 256
+        region = salt.salt_host_alloc(2 * len(slots) * step + 256)
+        try:
+            y = {}
+            for turn in range(2):
+                blobs = []
+                for i, sl in enumerate(slots):
+                    nb, at = r.blob_bytes(w.r_u[sl]), (turn * len(slots) + i) * step + shift
+                    blobs.append(r.make_blob(sl, version=10 * turn + i + 1, out=region.tensor[at:at + nb]))
+                r.build(stream=comp)
+                salt.salt_residual_load_batch(r.ctx, slots, blobs, side)
+                r.build(stream=comp)
+                xs = bf16_tensor(w.x(1))
+                y[turn] = bf16_tensor(w.y_in(1))
+                salt.salt_lora_apply(r.ctx, r.seg, 1, xs, y[turn], comp)
+            torch.cuda.synchronize()
+            assert r.device_error() == 0
+            assert salt.salt_guard_check(r.ctx, r.seg) == 0
+        finally:
+            torch.cuda.synchronize()
+            salt.salt_host_free(region)
+    for turn in range(2):
+        last = {sl: 10 * turn + i + 1 for i, sl in enumerate(slots)}
+        cents, res = oracle_tables(w, 1, version=lambda v: last.get(v, 0))
+        ref = oracle_mod.apply(w.x(1), w.y_in(1), w.dom_ids, w.slot_ids, cents, res)
+        assert_close(bf16_bits(y[turn]), ref, f"swap {turn} of {slots}")
