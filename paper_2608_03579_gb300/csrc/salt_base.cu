@@ -40,8 +40,8 @@
 //
 // Measured against one CTA per 128 x 128 tile with cp.async for x, no K
 // split and the shrink run to its end first: a 3B MLP layer at 8192 tokens
-// 2937 -> 890 us (1.41 PFLOP/s), an 8B layer at 512 tokens 746 -> 329 us, at
-// 24 tokens 552 -> 178 us.  x by TMA tile::gather4 instead of the gather
+// 2937 -> 890 us (1.41 PFLOP/s), an 8B layer at 512 tokens 746 -> 324 us, at
+// 24 tokens 552 -> 175 us.  x by TMA tile::gather4 instead of the gather
 // warps took 3050 us for the first (about 90 cycles a four-row copy).
 #include <cuda_bf16.h>
 
@@ -58,27 +58,29 @@ namespace {
 constexpr int BM = 128;                    // token rows per CTA (the UMMA M is BM * CG)
 constexpr int BK = 64;                     // K chunk (128-byte rows)
 constexpr int NST_MAX = 10;
-constexpr int BASE_RING = 208 * 1024;      // shared-memory ring
+constexpr int BASE_RING = 224 * 1024;      // shared-memory ring: 7 stages of a 256-column pair tile
 constexpr int BASE_THREADS = 384;
 constexpr int GW0 = 2, GWN = 6;            // gather warps; the ring holds at least as many stages (below)
 constexpr int EW0 = 8;                     // first epilogue warp
 constexpr int EPI_N = 128;
 constexpr int BAR_E = 1;                   // named barrier of the epilogue warps
-constexpr int MT_MAX = SALT_MAX_TOKENS / BM;
+constexpr int MT_MAX = SALT_MAX_TOKENS / (2 * BM);  // M tiles (of pairs: batches of one tile take CG = 1)
 constexpr int BASE_KS_MAX = 16;
 
 struct BaseInfo {
     uint64_t full[NST_MAX], empty[NST_MAX];
     uint64_t accf[2], acce[2];
-    int32_t ksteps[NST_MAX];               // a delta stage's K = 16 steps
     int32_t mt_b0[MT_MAX], mt_b1[MT_MAX];  // row blocks overlapping M tile: [b0, b1)
-    int32_t mt_nd[MT_MAX];                 // its delta chunks
-    int32_t mt_x0[MT_MAX];                 // its first token where this CTA's rows are consecutive tokens, else -1
+    uint32_t mt_nd[MT_MAX / 2];            // its delta chunks (at most 512), two tiles to a word
+    int16_t mt_x0[MT_MAX];                 // its first token where this CTA's rows are consecutive tokens, else -1
+    uint8_t ksteps[NST_MAX];               // a delta stage's K = 16 steps
     uint32_t tmem;
     int32_t last;
 };
-constexpr size_t BASE_SMEM = 1024 + BASE_RING + (sizeof(BaseInfo) + 127) / 128 * 128;
-static_assert(BASE_SMEM <= 227 * 1024, "shared memory exceeds the per-block limit");
+constexpr size_t BASE_SMEM = 1024 + BASE_RING + (sizeof(BaseInfo) + 15) / 16 * 16;
+// (an SM has 228 KB, of which it keeps 1 KB a CTA: room for a swap CTA beside)
+static_assert(BASE_SMEM + 2 * 1024 <= 228 * 1024, "shared memory exceeds what an SM has beside a swap CTA");
+static_assert(SALT_MAX_TOKENS <= 32767, "mt_x0 holds a token index");
 // A gather warp fills every GWN-th stage and waits only for its own slots'
 // phases; with at least GWN stages a slot's barrier is never two phases
 // behind the one it waits for (a parity wait could not tell).
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     for (int i = tid; i < n_mt; i += BASE_THREADS) {
         info.mt_b0[i] = 0x7fffffff;
         info.mt_b1[i] = 0;
-        info.mt_nd[i] = 0;
+        info.mt_nd[i >> 1] = 0;
     }
     __syncthreads();
     // Row blocks lie in grouped order and hold at most TM tokens, so each
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         for (int t = t0; t <= t1; ++t) {
             atomicMin(&info.mt_b0[t], b);
             atomicMax(&info.mt_b1[t], b + 1);
-            atomicAdd(&info.mt_nd[t], (S + BK - 1) / BK);
+            atomicAdd(&info.mt_nd[t >> 1], (uint32_t)((S + BK - 1) / BK) << (16 * (t & 1)));
         }
     }
     // Tiles whose rows are consecutive tokens (runs of a prefill batch) take x
@@ -195,7 +197,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             for (int i = lane; i < rows; i += 32) lin = lin && p.perm[m0 + i] == x0 + i;
             if (!__all_sync(0xffffffffu, lin)) x0 = -1;
         }
-        if (lane == 0) info.mt_x0[t] = x0;
+        if (lane == 0) info.mt_x0[t] = (int16_t)x0;
     }
     tc_fence_before();
     cta_or_cluster_sync<CG>();
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     // block run side by side, so W is read from memory about once), split u % KS
     auto chunk_lo = [&](int s) { return nk * s / KS; };
     const bool in_out = p.w_layout == SALT_W_IN_OUT;
-    auto n_delta = [&](int mt, int s) { const int nd = info.mt_nd[mt]; return nd > s ? (nd - s + KS - 1) / KS : 0; };
+    auto n_delta = [&](int mt, int s) { const int nd = (int)(info.mt_nd[mt >> 1] >> (16 * (mt & 1)) & 0xffffu); return nd > s ? (nd - s + KS - 1) / KS : 0; };
 
     if (warp == 0) {
         // ============================================================ TMA
@@ -293,7 +295,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     tc_fence_after();
                     const uint64_t xd = x0 + rp.slot * st16, wd = wmn0 + rp.slot * st16;
                             ok = __all_sync(0xffffffffu, ok);
-                    const int steps = ok ? *reinterpret_cast<volatile int32_t *>(&info.ksteps[rp.slot]) : 0;
+                    const int steps = ok ? *reinterpret_cast<volatile uint8_t *>(&info.ksteps[rp.slot]) : 0;
                     if (elect_one()) {
                         for (int kk = 0; kk < steps; ++kk)
                             umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, kk > 0 ? 1u : accum);
@@ -431,7 +433,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                             const bool in = sp != nullptr && col < p.d_out;
                             cp_async16(ws + (c >> 3) * 8192 + swz128(k, c & 7), in ? sp + col : p.x, in);
                         }
-                        if (lane == 0) info.ksteps[rp.slot] = kn >> 4;
+                        if (lane == 0) info.ksteps[rp.slot] = (uint8_t)(kn >> 4);
                         finish();
                         mine -= 1;  // this stage itself
                     }
