@@ -15,16 +15,19 @@
 //           V^T[S x M] (+)= Stack_A[S x chunk] * X[M x chunk]^T
 //       (tcgen05.mma, fp32 accumulator in tensor memory; the stack is the
 //       128-row operand, the tokens the N = 16..128 operand).  Each token
-//       keeps the centroid columns and its own user's columns.  With KS = 1
-//       the unit writes V_ext directly.  Otherwise every split stores an
-//       fp32 partial, waits (bounded) until all splits of the block have,
+//       keeps the centroid columns and its own user's columns.  Every split
+//       stores an fp32 partial, waits (bounded) until all splits of the block have,
 //       and then reduces its own slice of the token rows over the splits in
 //       split order (so the result does not depend on timing), writing
 //           V_ext[t,s] = s_c V[t,s]    for s < rc (centroid rows; s_c is the
 //                                      token's: the domain's scale times its gamma)
 //                      = s_u V[t,s]    for s in the token's own user's rows
 //                      = 0             otherwise
-//       as bf16.  Each unit then counts its rows as written.
+//       as bf16.  Each unit then counts its rows as written.  With more
+//       (block, projection) pairs than half the CTAs (prefill) K is not split:
+//       a whole unit computes V[M x S] (the tokens are the M operand, the
+//       stacks of one projection, or of all that read the same x, the N
+//       operand) and writes V_ext straight from the accumulator.
 //   expand items (row block, 64 output columns), cost-balanced over CTAs:
 //       Y[M x 64] += V_ext * Stack_B[:, cols] on the tensor cores (V_ext
 //       K-major, the B rows MN-major as they lie in memory, four fp32
@@ -248,8 +251,7 @@ constexpr int BAR_ALL = 4;                     // every thread (the inline unit 
 
 // The work of a shrink unit after its K loop, done by `nthr` threads
 // (warps first_warp .. first_warp + nthr/32 - 1, a whole number of groups of
-// four so that every TMEM lane quarter is read): with one split, V_ext
-// straight from the accumulator; otherwise the fp32 partial, the wait for
+// four so that every TMEM lane quarter is read): the fp32 partial, the wait for
 // the other splits of the block, the reduction of this unit's slice of the
 // token rows over the splits (in split order) and the V rows written.  Then
 // the unit's rows are counted as written.  The shrink tables of the unit
