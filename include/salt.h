@@ -294,8 +294,9 @@ salt_status salt_residual_load(salt_ctx *ctx, int32_t slot, const void *host_blo
  * salt_residual_load before anything is enqueued (an error leaves every
  * slot as it was).  On side_stream: one wait for the applies enqueued so
  * far on every segments object that refers to any of the slots, then the
- * blobs: by one kernel that reads them from host memory (four or more, all in
- * salt_host_alloc memory on 16-byte boundaries, the slots distinct) and one
+ * blobs: by one kernel that reads them from host memory (four or more of at
+ * most 4 MB, all in salt_host_alloc memory on 16-byte boundaries, the slots
+ * distinct) and one
  * ready event, else by one cudaMemcpyAsync per blob, each followed by its
  * slot's ready event.  The result is that of n salt_residual_load calls in
  * order.  n == 0 does nothing.

@@ -417,9 +417,13 @@ void slot_loaded(salt_ctx *ctx, int32_t slot, int32_t rank, int32_t batch)
     ctx->slot_seq[slot] += 1;
 }
 
-// Loads of one launch: at least this many blobs, in library host regions.
-// (A single blob is one copy-engine copy, 6.5 us for 1.31 MB.)
+// Loads of one launch: at least this many blobs, in library host regions,
+// none larger than SWAP_LAUNCH_BYTES.  (A single blob is one copy-engine copy,
+// 6.5 us for 1.31 MB; between two copies the engine pays 2 us, which large
+// ones make up: a 32-layer 8B step with 64 blobs of 10.5 MB ran 3.32 ms by
+// copies and 3.70 by the launch, a four-layer one with 1.31 MB blobs 538 and 458 us.)
 constexpr int SWAP_LAUNCH_MIN = 4;
+constexpr uint64_t SWAP_LAUNCH_BYTES = 4 << 20;
 
 // The loads of n checked blobs on `side`: readers first (every segments
 // object that names one of the slots waits for its uses, once), then the
@@ -439,7 +443,8 @@ salt_status enqueue_loads(salt_ctx *ctx, int32_t n, const int32_t *slots, const 
     }
     bool launch = n >= SWAP_LAUNCH_MIN && ctx->direct_host;
     for (int32_t i = 0; i < n && launch; ++i)
-        launch = (reinterpret_cast<uintptr_t>(blobs[i]) & 15) == 0 && (bytes[i] & 15) == 0 && in_host_region(blobs[i], bytes[i]);
+        launch = (reinterpret_cast<uintptr_t>(blobs[i]) & 15) == 0 && (bytes[i] & 15) == 0 && bytes[i] <= SWAP_LAUNCH_BYTES &&
+                 in_host_region(blobs[i], bytes[i]);
     if (launch) {  // (a slot named twice is loaded in order, by copies)
         std::vector<int32_t> sorted(slots, slots + n);
         std::sort(sorted.begin(), sorted.end());
