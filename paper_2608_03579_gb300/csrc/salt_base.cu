@@ -73,7 +73,9 @@ struct BaseInfo {
     int32_t mt_b0[MT_MAX], mt_b1[MT_MAX];  // row blocks overlapping M tile: [b0, b1)
     uint32_t mt_nd[MT_MAX / 2];            // its delta chunks (at most 512), two tiles to a word
     int16_t mt_x0[MT_MAX];                 // its first token where this CTA's rows are consecutive tokens, else -1
+    uint32_t mt_peer[MT_MAX / 32];         // bit: the pair's second CTA gathers the tile's rows
     uint8_t ksteps[NST_MAX];               // a delta stage's K = 16 steps
+    alignas(16) uint32_t token[4];         // copied by the second CTA's gather warps to signal the first
     uint32_t tmem;
     int32_t last;
 };
@@ -156,7 +158,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     }
     if (tid == 0) {
         for (int i = 0; i < NST_MAX; ++i) {
-            mbar_init(bar(info.full[i]), 2 * CG);  // per CTA: the TMA warp and a gather warp
+            mbar_init(bar(info.full[i]), 1 + CG);  // the TMA warps and the first CTA's gather warp
             mbar_init(bar(info.empty[i]), 1);
         }
         for (int i = 0; i < 2; ++i) {
@@ -169,6 +171,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         info.mt_b0[i] = 0x7fffffff;
         info.mt_b1[i] = 0;
         info.mt_nd[i >> 1] = 0;
+        info.mt_peer[i >> 5] = 0;
     }
     __syncthreads();
     // Row blocks lie in grouped order and hold at most TM tokens, so each
@@ -189,15 +192,18 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     // Tiles whose rows are consecutive tokens (runs of a prefill batch) take x
     // by plain TMA tiles; a batch of one tile is not looked at.
     for (int t = warp; t < n_mt; t += BASE_THREADS / 32) {
-        const int m0 = (t * CG + rank) * BM, rows = min(BM, T - m0);
-        int x0 = -1;
-        if (CG == 2 && rows > 0) {
-            x0 = p.perm[m0];
-            bool lin = true;
-            for (int i = lane; i < rows; i += 32) lin = lin && p.perm[m0 + i] == x0 + i;
-            if (!__all_sync(0xffffffffu, lin)) x0 = -1;
+        for (int h = rank; h < CG; ++h) {  // the first CTA looks at both halves
+            const int m0 = (t * CG + h) * BM, rows = min(BM, T - m0);
+            int x0 = -1;
+            if (CG == 2 && rows > 0) {
+                x0 = p.perm[m0];
+                bool lin = true;
+                for (int i = lane; i < rows; i += 32) lin = lin && p.perm[m0 + i] == x0 + i;
+                if (!__all_sync(0xffffffffu, lin)) x0 = -1;
+            }
+            if (lane == 0 && h == rank) info.mt_x0[t] = (int16_t)x0;
+            if (lane == 0 && h == 1 && x0 < 0) atomicOr(&info.mt_peer[t >> 5], 1u << (t & 31));
         }
-        if (lane == 0) info.mt_x0[t] = (int16_t)x0;
     }
     tc_fence_before();
     cta_or_cluster_sync<CG>();
@@ -206,6 +212,11 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     bool ok = true;  // a bounded wait gave up: no further waits, no further loads
     auto wait_bar = [&](const uint64_t &b, uint32_t parity) {
         if (ok && !mbar_wait(smem_u32(&b), parity)) ok = false;
+    };
+    // a stage; peer: a thread of the pair's second CTA staged some of it
+    auto wait_full = [&](uint32_t slot, uint32_t parity, bool peer) {
+        const uint32_t b = smem_u32(&info.full[slot]);
+        if (ok && !(peer ? mbar_wait_cluster<CG>(b, parity) : mbar_wait(b, parity))) ok = false;
     };
     // unit u: tile u / KS (M tile tile % n_mt: the M tiles of one W column
     // block run side by side, so W is read from memory about once), split u % KS
@@ -228,6 +239,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         for (int u = cl; u < n_units && ok; u += n_cl) {
             const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
             const int k1 = chunk_lo(s + 1), x0 = info.mt_x0[mt];
+            const bool peer = CG == 2 && rank == 0 && (info.mt_peer[mt >> 5] >> (mt & 31) & 1u);
             for (int kc = chunk_lo(s); kc < k1 && ok; ++kc, advance()) {
                 next_slot();
                 if (!ok) break;
@@ -235,7 +247,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     const uint32_t ws = ring32 + rp.slot * stage + x_bytes;
                     const uint32_t fb = leader_addr<CG>(bar(info.full[rp.slot]));
                     const int k0 = kc * BK;
-                    mbar_expect_tx_cluster<CG>(fb, (uint32_t)NB * 128u + (x0 >= 0 ? x_bytes : 0u));
+                    mbar_expect_tx_cluster<CG>(fb, (uint32_t)NB * 128u + (x0 >= 0 ? x_bytes : 0u) + (peer ? BULK_SIGNAL_BYTES : 0u));
                     if (x0 >= 0) tma_load_2d_cg<CG>(ws - x_bytes, &p.xmap, k0, x0, fb);
                     if (in_out) {
                         // W[d_in][d_out]: boxes of 64 K rows x 64 N columns (MN-major)
@@ -250,7 +262,11 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             // the delta's stages hold nothing of W
             for (int j = n_delta(mt, s); j > 0 && ok; --j, advance()) {
                 next_slot();
-                if (ok && elect_one()) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
+                if (ok && elect_one()) {
+                    const uint32_t fb = leader_addr<CG>(bar(info.full[rp.slot]));
+                    if (CG == 2 && rank == 0) mbar_expect_tx_cluster<CG>(fb, BULK_SIGNAL_BYTES);
+                    else mbar_arrive_relaxed_cluster<CG>(fb);
+                }
                 __syncwarp();
             }
         }
@@ -277,8 +293,9 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                 if (lt >= 2) wait_bar(info.acce[buf], ((lt - 2) >> 1) & 1);
                 tc_fence_after();
                 uint32_t accum = 0;
+                const bool peer = CG == 2 && (info.mt_peer[mt >> 5] >> (mt & 31) & 1u);
                 for (int n = chunk_lo(s + 1) - chunk_lo(s); n > 0; --n, rp.advance(1, nst)) {
-                    wait_bar(info.full[rp.slot], rp.phase);
+                    wait_full(rp.slot, rp.phase, peer);
                     tc_fence_after();
                     const uint64_t xd = x0 + rp.slot * st16, wd = w0 + rp.slot * st16;
                     if (elect_one()) {
@@ -291,7 +308,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     accum = 1;
                 }
                 for (int n = n_delta(mt, s); n > 0; --n, rp.advance(1, nst)) {
-                    wait_bar(info.full[rp.slot], rp.phase);
+                    wait_full(rp.slot, rp.phase, CG == 2);
                     tc_fence_after();
                     const uint64_t xd = x0 + rp.slot * st16, wd = wmn0 + rp.slot * st16;
                             ok = __all_sync(0xffffffffu, ok);
@@ -311,7 +328,9 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         __syncwarp();
     } else if (warp < EW0) {
         // ============================================================ gathers
-        // Stage g (counted over the CTA's units) belongs to warp g % GWN.
+        // Stage g (counted over the CTA's units) belongs to warp g % GWN.  The
+        // first CTA's warps arrive on the stage's barrier, the second one's
+        // add BULK_SIGNAL_BYTES to the bytes that it waits for.
         const int w = warp - GW0;
         RingPos rp;                 // the warp's next stage
         rp.advance(w, nst);
@@ -332,7 +351,10 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             cp_async_wait<0>();
             fence_async_smem();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
+            if (lane == 0) {
+                if (rank == 0) mbar_arrive_release(bar(info.full[rp.slot]));
+                else bulk_signal_leader(smem_u32(info.token), bar(info.full[rp.slot]));
+            }
             next_stage();
         };
         uint32_t xoff[BM / 4];      // this lane's token rows (row 4 i + lane / 8), in 16-byte units of x
@@ -359,7 +381,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                 begin();
                 if (!ok) break;
                 if (lin) {  // the TMA warp loads the rows
-                    if (lane == 0) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.full[rp.slot])));
+                    if (lane == 0 && rank == 0) mbar_arrive_relaxed(bar(info.full[rp.slot]));
                     next_stage();
                     continue;
                 }

@@ -133,3 +133,30 @@ def test_with_base_tile_edges(salt_lib, oracle_mod, wl, layout, T, d_in, d_out):
         assert salt_lib.salt_guard_check(r.ctx, r.seg) == 0
     assert np.array_equal(got, again)
     assert_close(got, _ref(oracle_mod, w, 0, W, layout), f"with base, {T} x {d_in} x {d_out}, layout {layout}")
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+def test_with_base_pairs_repeat(salt_lib, oracle_mod, wl, layout):
+    """CTA pairs whose second CTA gathers its rows (users in random order), a
+    K loop of several rounds of the ring and delta chunks: every run gives
+    the same bits, so no stage is read before the other CTA's copies landed."""
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
+    T, n_users, d_in, d_out = 512, 64, 2048, 512
+    u = (wl.uniform(33, 1, T) * n_users).astype(np.int32) % n_users
+    w = wl.Workload("base_repeat", 33, [("p", d_in, d_out)], 2, [64, 5], n_users, [1, 2] * (n_users // 2),
+                    dom_ids=(u % 2).astype(np.int32), slot_ids=u)
+    w.y_mode = "zeros"
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        r.build()
+        W = _weight(wl, 33, d_in, d_out, layout)
+        x, Wd = bf16_tensor(w.x(0)), bf16_tensor(W)
+        ys = [torch.full((T, d_out), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(20)]
+        for y in ys:
+            salt_lib.salt_lora_apply_with_base(r.ctx, r.seg, 0, x, Wd, layout, y)
+        torch.cuda.synchronize()
+        assert r.device_error() == 0
+    first = bf16_bits(ys[0])
+    assert all(np.array_equal(first, bf16_bits(y)) for y in ys[1:])
+    assert_close(first, _ref(oracle_mod, w, 0, W, layout), f"with base, repeated, layout {layout}")
