@@ -66,6 +66,8 @@ constexpr int EPI_N = 128;
 constexpr int BAR_E = 1;                   // named barrier of the epilogue warps
 constexpr int MT_MAX = SALT_MAX_TOKENS / (2 * BM);  // M tiles (of pairs: batches of one tile take CG = 1)
 constexpr int BASE_KS_MAX = 16;
+constexpr int SPLIT_POLLS = 128;           // a split's wait for the others of its tile
+static_assert(BASE_KS_MAX <= 16, "a split is a bit of half a counter word");
 
 struct BaseInfo {
     uint64_t full[NST_MAX], empty[NST_MAX];
@@ -77,7 +79,7 @@ struct BaseInfo {
     uint8_t ksteps[NST_MAX];               // a delta stage's K = 16 steps
     alignas(16) uint32_t token[4];         // copied by the second CTA's gather warps to signal the first
     uint32_t tmem;
-    int32_t last;
+    uint32_t shares;
 };
 constexpr size_t BASE_SMEM = 1024 + BASE_RING + (sizeof(BaseInfo) + 15) / 16 * 16;
 // (an SM has 228 KB, of which it keeps 1 KB a CTA: room for a swap CTA beside)
@@ -467,7 +469,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         const int q = warp & 3, row = q * 32 + lane, et = tid - 32 * EW0;
         const bool wide = (p.d_out & 15) == 0 && (reinterpret_cast<uintptr_t>(p.y) & 31) == 0;
         uint32_t lt = 0;
-        const bool share = n_units <= n_cl;
+        const bool share = n_units <= n_cl;  // one unit a CTA
         if (KS > 1) pdl_wait();  // the partials' workspace is the shrink's
         for (int u = cl; u < n_units; u += n_cl, ++lt) {
             const int tile = u / KS, mt = tile % n_mt, n0 = tile / n_mt * BN;
@@ -510,85 +512,93 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
             __syncwarp();
             if (lane == 0) mbar_arrive_relaxed_cluster<CG>(leader_addr<CG>(bar(info.acce[buf])));
             if (KS == 1) continue;
-            // Sum the partials of the tile (this CTA's rows) in split order.
-            // When every unit has its own CTAs at once, each split waits
-            // (bounded) for the others and sums its share; otherwise the
-            // split that finishes last sums them all.
+            // Sum the partials of the tile (this CTA's rows) in split order, a
+            // share of them per split.  ctr[0] counts the splits stored (low
+            // half) and marks the ones that left their share to the split
+            // that stores last (high half).  Where every unit may run at once
+            // a split waits a while for the others (about 0.1 ms) and then
+            // leaves; so nothing depends on the CTAs of a tile running
+            // together, which other streams' launches can prevent.  (Leaving
+            // at once: an 8B layer at 24 tokens 195 us, 175 with the wait.)
             __threadfence();
             named_sync(BAR_E, EPI_N);
             uint32_t *ctr = p.ctr + 2 * (tile * CG + rank);
             if (et == 0) {
-                const uint32_t n = atomicAdd(ctr, 1u) + 1u;
-                bool go = n == (uint32_t)KS;
-                if (share) {
-                    for (int i = 0; i < (1 << 22) && !go; ++i) {
-                        uint32_t c;
+                const uint32_t own = 1u << (u - tile * KS);
+                uint32_t c = atomicAdd(ctr, 1u), sum = own;
+                if ((c & 0xffffu) + 1u == (uint32_t)KS) {
+                    sum |= c >> 16;
+                } else {
+                    bool all = false;
+                    for (int i = 0; i < SPLIT_POLLS && share && !all; ++i) {
                         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(c) : "l"(ctr) : "memory");
-                        go = c == (uint32_t)KS;
-                        if (!go) __nanosleep(32);
+                        all = (c & 0xffffu) == (uint32_t)KS;
+                        if (!all) __nanosleep(32);
                     }
-                    if (!go) ok = false;
-                    go = true;
-                } else if (go) {
-                    atomicExch(ctr, 0u);  // zero for the next launch
+                    if (!all && (atomicOr(ctr, own << 16) & 0xffffu) != (uint32_t)KS) sum = 0u;
                 }
-                info.last = go;
+                info.shares = sum;
                 __threadfence();
             }
             named_sync(BAR_E, EPI_N);
-            if (!info.last) continue;
+            const uint32_t shares = info.shares;
+            if (!shares) continue;
             const float *p0 = p.part + ((int64_t)tile * KS * CG + rank) * (m_rows * BN);
             const int64_t ps = (int64_t)CG * m_rows * BN;
-            const int lc = BN == 256 ? 5 : 4, n_all = rows << lc, s_own = u - tile * KS;
-            const int n_it = share ? n_all * (s_own + 1) / KS : n_all;
-            // (row, 8 columns) items, two a round per thread, up to four splits' loads in flight
-            for (int base = (share ? n_all * s_own / KS : 0) + et; base < n_it; base += 2 * EPI_N) {
-                float a[2][8] = {};
-                for (int s0 = 0; s0 < KS; s0 += 4) {
-                    float4 v[2][4][2];
+            const int lc = BN == 256 ? 5 : 4, n_all = rows << lc;
+            // consecutive shares together
+            for (uint32_t left = shares; left;) {
+                const int s0 = __ffs(left) - 1, n = __ffs(~(left >> s0)) - 1, n_it = n_all * (s0 + n) / KS;
+                left &= ~(((1u << n) - 1u) << s0);
+                // (row, 8 columns) items, two a round per thread, up to four splits' loads in flight
+                for (int base = n_all * s0 / KS + et; base < n_it; base += 2 * EPI_N) {
+                    float a[2][8] = {};
+                    for (int k0 = 0; k0 < KS; k0 += 4) {
+                        float4 v[2][4][2];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h)
+                        for (int h = 0; h < 2; ++h)
 #pragma unroll
-                        for (int s = 0; s < 4; ++s) {
-                            const int it = base + h * EPI_N;
-                            if (it < n_it && s0 + s < KS) {
-                                const int c8 = it & ((1 << lc) - 1), r = it >> lc;
-                                const float4 *src = reinterpret_cast<const float4 *>(p0 + (s0 + s) * ps + (c8 * m_rows + r) * 8);
-                                v[h][s][0] = __ldcg(src);
-                                v[h][s][1] = __ldcg(src + 1);
-                            } else {
-                                v[h][s][0] = v[h][s][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            for (int s = 0; s < 4; ++s) {
+                                const int it = base + h * EPI_N;
+                                if (it < n_it && k0 + s < KS) {
+                                    const int c8 = it & ((1 << lc) - 1), r = it >> lc;
+                                    const float4 *src = reinterpret_cast<const float4 *>(p0 + (k0 + s) * ps + (c8 * m_rows + r) * 8);
+                                    v[h][s][0] = __ldcg(src);
+                                    v[h][s][1] = __ldcg(src + 1);
+                                } else {
+                                    v[h][s][0] = v[h][s][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                }
                             }
-                        }
 #pragma unroll
-                    for (int h = 0; h < 2; ++h)
+                        for (int h = 0; h < 2; ++h)
 #pragma unroll
-                        for (int s = 0; s < 4; ++s) {
-                            a[h][0] += v[h][s][0].x;
-                            a[h][1] += v[h][s][0].y;
-                            a[h][2] += v[h][s][0].z;
-                            a[h][3] += v[h][s][0].w;
-                            a[h][4] += v[h][s][1].x;
-                            a[h][5] += v[h][s][1].y;
-                            a[h][6] += v[h][s][1].z;
-                            a[h][7] += v[h][s][1].w;
-                        }
-                }
+                            for (int s = 0; s < 4; ++s) {
+                                a[h][0] += v[h][s][0].x;
+                                a[h][1] += v[h][s][0].y;
+                                a[h][2] += v[h][s][0].z;
+                                a[h][3] += v[h][s][0].w;
+                                a[h][4] += v[h][s][1].x;
+                                a[h][5] += v[h][s][1].y;
+                                a[h][6] += v[h][s][1].z;
+                                a[h][7] += v[h][s][1].w;
+                            }
+                    }
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int it = base + h * EPI_N;
-                    if (it >= n_it) continue;
-                    const int r = it >> lc, col = n0 + (it & ((1 << lc) - 1)) * 8;
-                    if (col < p.d_out)
-                        *reinterpret_cast<uint4 *>(p.y + (int64_t)p.perm[m0 + r] * p.d_out + col) =
-                            make_uint4(pack_bf16(a[h][0], a[h][1]), pack_bf16(a[h][2], a[h][3]),
-                                       pack_bf16(a[h][4], a[h][5]), pack_bf16(a[h][6], a[h][7]));
+                    for (int h = 0; h < 2; ++h) {
+                        const int it = base + h * EPI_N;
+                        if (it >= n_it) continue;
+                        const int r = it >> lc, col = n0 + (it & ((1 << lc) - 1)) * 8;
+                        if (col < p.d_out)
+                            *reinterpret_cast<uint4 *>(p.y + (int64_t)p.perm[m0 + r] * p.d_out + col) =
+                                make_uint4(pack_bf16(a[h][0], a[h][1]), pack_bf16(a[h][2], a[h][3]),
+                                           pack_bf16(a[h][4], a[h][5]), pack_bf16(a[h][6], a[h][7]));
+                    }
                 }
             }
-            if (share) {
-                // the last split to have read the partials zeroes the counters
-                named_sync(BAR_E, EPI_N);
-                if (et == 0 && atomicAdd(ctr + 1, 1u) + 1u == (uint32_t)KS) {
+            // every share summed: zero for the next launch
+            if (et == 0) {
+                const uint32_t n = __popc(shares);
+                if (atomicAdd(ctr + 1, n) + n == (uint32_t)KS) {
                     atomicExch(ctr, 0u);
                     atomicExch(ctr + 1, 0u);
                 }

@@ -160,3 +160,38 @@ def test_with_base_pairs_repeat(salt_lib, oracle_mod, wl, layout):
     first = bf16_bits(ys[0])
     assert all(np.array_equal(first, bf16_bits(y)) for y in ys[1:])
     assert_close(first, _ref(oracle_mod, w, 0, W, layout), f"with base, repeated, layout {layout}")
+
+
+@pytest.mark.parametrize("T,d_in,d_out", [(24, 4096, 4096), (24, 8192, 1032), (200, 14336, 2048)])
+def test_with_base_splits_on_two_streams(salt_lib, oracle_mod, wl, T, d_in, d_out):
+    """K-split launches of two segments objects on two streams: the CTAs of a
+    tile need not run together, so every result is the same bits as alone."""
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
+    salt, n_users = salt_lib, 16
+    u = (wl.uniform(35, 1, T) * n_users).astype(np.int32) % n_users
+    w = wl.Workload("base_streams", 35, [("p", d_in, d_out)], 2, [64, 5], n_users, [1, 2] * (n_users // 2),
+                    dom_ids=(u % 2).astype(np.int32), slot_ids=u)
+    w.y_mode = "zeros"
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        segs = [r.seg, salt.salt_segments_create(r.ctx)]
+        try:
+            for seg in segs:
+                salt.salt_build_segments(r.ctx, seg, w.dom_ids, w.slot_ids)
+            x, Wd = bf16_tensor(w.x(0)), bf16_tensor(_weight(wl, 35, d_in, d_out, 1))
+            ys = [torch.full((T, d_out), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(41)]
+            salt.salt_lora_apply_with_base(r.ctx, r.seg, 0, x, Wd, 1, ys[0])
+            streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+            torch.cuda.synchronize()
+            for i, y in enumerate(ys[1:]):
+                salt.salt_lora_apply_with_base(r.ctx, segs[i & 1], 0, x, Wd, 1, y, streams[i & 1])
+            torch.cuda.synchronize()
+            assert r.device_error() == 0
+            for seg in segs:
+                assert salt.salt_guard_check(r.ctx, seg) == 0
+        finally:
+            salt.salt_segments_destroy(segs[1])
+    first = bf16_bits(ys[0])
+    assert all(np.array_equal(first, bf16_bits(y)) for y in ys[1:])
+    assert_close(first, _ref(oracle_mod, w, 0, _weight(wl, 35, d_in, d_out, 1), 1), f"two streams, {T} x {d_in} x {d_out}")
