@@ -89,6 +89,7 @@ typedef enum salt_status {
 #define SALT_DEVERR_RANK 0x10u
 #define SALT_DEVERR_TIMEOUT 0x20u        /* a bounded in-kernel wait gave up (results of that call invalid) */
 #define SALT_DEVERR_GAMMA_RANGE 0x40u
+#define SALT_DEVERR_BATCH 0x80u          /* a captured salt_lora_apply_with_base was replayed on a larger batch */
 
 /*
  * Context configuration.  d_in / d_out are host arrays of n_layers entries,
@@ -417,7 +418,10 @@ salt_status salt_lora_apply_grouped(salt_ctx *ctx, const salt_segments *seg, int
  * 128-token tiles in grouped order and adds each overlapping row block's
  * V * [B_c; b_u] into the same accumulator.  Asynchronous; the workspace
  * is shared with salt_lora_apply on the same segments object (stream
- * order keeps them apart).
+ * order keeps them apart).  A captured call may be replayed after the
+ * segments object was rebuilt with at most as many tokens as it had at the
+ * capture (y rows of tokens outside the new batch are not touched); of a
+ * larger batch it computes and writes nothing and raises SALT_DEVERR_BATCH.
  */
 salt_status salt_lora_apply_with_base(salt_ctx *ctx, const salt_segments *seg, int32_t layer,
                                       const void *x, const void *W, int32_t layout, void *y,

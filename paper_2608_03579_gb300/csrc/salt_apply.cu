@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(APPLY_THREADS, 1) salt_apply_kernel(const __gr
     // dependency wait) only once everything before this launch is complete.
     if (!p.shrink_only) pdl_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n_blk = min(p.counts[3], p.w.blk_cap);
+    const int n_blk = p.shrink_only && p.counts[0] > p.max_tok ? 0 : min(p.counts[3], p.w.blk_cap);
     if (p.counts[3] > p.w.blk_cap && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(p.err, SALT_DEVERR_RANK);
     const int nu = p.n_unit_prefix[p.n_proj];
     if (n_blk <= 0 || nu <= 0) {  // the same for every CTA

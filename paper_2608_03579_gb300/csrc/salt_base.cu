@@ -141,14 +141,17 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = CG == 2 ? (int)cluster_ctarank() : 0;  // this CTA's half of the tile
     const int cl = blockIdx.x / CG, n_cl = gridDim.x / CG;
-    const int T = p.T, BN = p.bn, NB = BN / CG;             // NB: W columns this CTA loads
+    // The batch as built last: a captured launch is replayed on later ones.
+    // The launch is shaped for up to p.T tokens; of more it computes nothing.
+    const int T = p.counts[0] <= p.T ? p.counts[0] : 0;
+    const int BN = p.bn, NB = BN / CG;                      // NB: W columns this CTA loads
     const int n_mt = (T + BM * CG - 1) / (BM * CG), n_nt = (p.d_out + BN - 1) / BN;
     const int KS = p.ks, n_units = n_mt * n_nt * KS;
     const int nk = (p.d_in + BK - 1) / BK;
     // a stage: the CTA's token rows (only as many as the batch can fill),
     // then its W columns.  The UMMA reads 128 rows: with fewer loaded the
     // rest are whatever follows, and reach only accumulator rows past T.
-    const int m_rows = CG == 2 ? BM : (min(T, BM) + 15) & ~15;
+    const int m_rows = CG == 2 ? BM : (min(p.T, BM) + 15) & ~15;
     const uint32_t x_bytes = (uint32_t)m_rows * 128u, stage = x_bytes + (uint32_t)NB * 128u;
     const uint32_t nst = min((uint32_t)NST_MAX, (uint32_t)BASE_RING / stage);
     auto bar = [](const uint64_t &b) { return smem_u32(&b); };
@@ -158,6 +161,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         tmem_alloc<CG>(smem_u32(&info.tmem), 2 * BN);
         tmem_relinquish<CG>();
     }
+    if (p.counts[0] > p.T && blockIdx.x == 0 && tid == 0) atomicOr(p.err, SALT_DEVERR_BATCH);
     if (tid == 0) {
         for (int i = 0; i < NST_MAX; ++i) {
             mbar_init(bar(info.full[i]), 1 + CG);  // the TMA warps and the first CTA's gather warp
@@ -184,7 +188,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         const int4 r = *reinterpret_cast<const int4 *>(p.blk + BLK_INTS * b);
         const int S = r.w + p.blk[BLK_INTS * b + BLK_NRES];
         if (S <= 0 || S > S_MAX || r.y <= 0) continue;  // flagged by the shrink
-        const int t0 = r.x / (BM * CG), t1 = (r.x + r.y - 1) / (BM * CG);
+        const int t0 = r.x / (BM * CG), t1 = min((r.x + r.y - 1) / (BM * CG), n_mt - 1);
         for (int t = t0; t <= t1; ++t) {
             atomicMin(&info.mt_b0[t], b);
             atomicMax(&info.mt_b1[t], b + 1);

@@ -164,6 +164,7 @@ struct ApplyParams {
     int32_t tok_c4;      // 4-column pieces of a partial row that can hold anything (rc_max + r_max columns)
     uint32_t tok_c4_inv; // floor(2^32 / tok_c4) + 1: divides numbers below 2^12 by it (tok_c4 > 1)
     int32_t shrink_only; // write the V tiles of the row blocks and stop (the base-weight kernel expands)
+    int32_t max_tok;     // shrink_only: the tokens the base launch is shaped for; nothing is done for a larger batch
     const uint8_t *pool;
     int64_t slot_stride;
     ApplyWork w;
@@ -192,7 +193,8 @@ struct BaseParams {
     int64_t res_off;         // sum over earlier layers of (d_in + d_out), in elements
     float *part;             // fp32 partials of the K splits (the apply's partial tiles)
     uint32_t *ctr;           // [BASE_CTRS] splits stored and summed, per (tile, CTA of the pair); zero between launches
-    int32_t T, d_in, d_out, rc_max, w_layout, blk_cap;
+    int32_t T;               // tokens the launch is shaped for (the batch's own count is counts[0])
+    int32_t d_in, d_out, rc_max, w_layout, blk_cap;
     int32_t bn, ks;          // tile columns and K splits (launch_base)
     uint32_t *err;
 };

@@ -1283,6 +1283,7 @@ salt_status apply_grouped(salt_ctx *ctx, const salt_segments *seg_, int32_t n, c
     p.w = seg->work;
     p.err = ctx->err_dev;
     p.shrink_only = shrink_only ? 1 : 0;
+    p.max_tok = seg->T;
     const int ctas = shrink_only ? base_shrink_ctas(seg->T, p.proj[0].d_in, p.proj[0].d_out, seg->n_blk_est) : 0;
     // The first apply after a build waits for the segment kernel in full;
     // later ones overlap their table reads with the previous kernel.

@@ -195,3 +195,50 @@ def test_with_base_splits_on_two_streams(salt_lib, oracle_mod, wl, T, d_in, d_ou
     first = bf16_bits(ys[0])
     assert all(np.array_equal(first, bf16_bits(y)) for y in ys[1:])
     assert_close(first, _ref(oracle_mod, w, 0, _weight(wl, 35, d_in, d_out, 1), 1), f"two streams, {T} x {d_in} x {d_out}")
+
+
+@pytest.mark.parametrize("T,later", [
+    (40, (17, 1, 0, 40, 41, 500, 11000, 33)),       # one CTA a tile; replayed on up to 86 tiles' worth of tokens
+    (300, (130, 257, 20, 300, 301, 8200, 16384, 299)),  # pairs
+])
+def test_with_base_replayed_after_rebuilds(salt_lib, oracle_mod, wl, T, later):
+    """A captured call replayed after rebuilds: batches up to the capture's
+    are computed whole, other rows of y stay; a larger one raises a flag and
+    leaves y alone, and the next replay is right again."""
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
+    n_users, d_in, d_out, T_max = 24, 1032, 392, 16384
+    u = (wl.uniform(37, 1, T_max) * n_users).astype(np.int32) % n_users
+    w = wl.Workload("base_replay", 37, [("p", d_in, d_out)], 2, [64, 5], n_users, [1, 2] * (n_users // 2),
+                    dom_ids=(u % 2).astype(np.int32), slot_ids=u)
+    w.y_mode = "zeros"
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        W = _weight(wl, 37, d_in, d_out, 1)
+        x, Wd = bf16_tensor(w.x(0)), bf16_tensor(W)
+        y = torch.empty(T_max, d_out, dtype=torch.bfloat16, device="cuda")
+        s = torch.cuda.Stream()
+        r.build(w.dom_ids[:T], w.slot_ids[:T], stream=s)
+        salt_lib.salt_lora_apply_with_base(r.ctx, r.seg, 0, x, Wd, 1, y, s)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            salt_lib.salt_lora_apply_with_base(r.ctx, r.seg, 0, x, Wd, 1, y, s)
+        cents, res = oracle_tables(w, 0)
+        for n in later:
+            # the last n tokens' ids for the first n tokens: another grouping than at the capture
+            dom, slot = w.dom_ids[T_max - n:], w.slot_ids[T_max - n:]
+            r.build(dom, slot, stream=s)
+            y.fill_(7.0)
+            torch.cuda.synchronize()
+            with torch.cuda.stream(s):
+                g.replay()
+            torch.cuda.synchronize()
+            got = bf16_bits(y)
+            assert salt_lib.salt_guard_check(r.ctx, r.seg) == 0
+            assert r.device_error() == (0x80 if n > T else 0), n
+            done = n if n <= T else 0
+            assert (got[done:] == 0x40E0).all(), f"{n} tokens: rows past the batch were written"
+            if done:
+                ref = oracle_mod.apply(w.x(0)[:n], None, dom, slot, cents, res, w_base=W, w_layout=1)
+                assert_close(got[:n], ref, f"captured on {T} tokens, replayed on {n}")
