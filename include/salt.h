@@ -427,6 +427,19 @@ salt_status salt_lora_apply_with_base(salt_ctx *ctx, const salt_segments *seg, i
                                       const void *x, const void *W, int32_t layout, void *y,
                                       salt_stream_t stream);
 
+/* How salt_lora_apply_with_base would launch the GEMM of `layer` for the batch
+ * seg was built from last (diagnostics; no device work; all zero for an empty
+ * batch). */
+typedef struct salt_base_shape {
+    int32_t cta_group;    /* CTAs sharing a tile: 1 (128 tokens) or 2 (256 tokens) */
+    int32_t tile_cols;    /* output columns of a tile */
+    int32_t k_splits;     /* splits of d_in per tile */
+    int32_t shrink_ctas;  /* CTAs of the shrink beside the K loop (0: every SM, before it) */
+    int32_t units;        /* (tile, split) units */
+    int32_t clusters;     /* CTAs or CTA pairs they are spread over */
+} salt_base_shape;
+salt_status salt_base_get_shape(salt_ctx *ctx, const salt_segments *seg, int32_t layer, salt_base_shape *shape);
+
 /*
  * salt_lora_apply for callers that cannot allocate device memory when they
  * apply - for example a serving engine whose device memory is planned up

@@ -717,6 +717,21 @@ int base_shrink_ctas(int T, int d_in, int d_out, int n_blk)
     return plan_here(T, d_in, d_out, n_blk, &pl, &n_cl) ? pl.shrink_ctas : 0;
 }
 
+bool base_launch_shape(int T, int d_in, int d_out, int n_blk, salt_base_shape *out)
+{
+    BasePlan pl;
+    int max_cl;
+    if (!plan_here(T, d_in, d_out, n_blk, &pl, &max_cl)) return false;
+    const int bm = BM * pl.cg;
+    out->cta_group = pl.cg;
+    out->tile_cols = pl.bn;
+    out->k_splits = pl.ks;
+    out->shrink_ctas = pl.shrink_ctas;
+    out->units = ((T + bm - 1) / bm) * ((d_out + pl.bn - 1) / pl.bn) * pl.ks;
+    out->clusters = std::min(out->units, max_cl);
+    return true;
+}
+
 cudaError_t launch_base(BaseParams &p, const uint16_t *W, int n_blk, cudaStream_t stream)
 {
     BasePlan pl;

@@ -206,6 +206,8 @@ cudaError_t base_prepare(int device);
 cudaError_t launch_base(BaseParams &p, const uint16_t *W, int n_blk, cudaStream_t stream);
 // CTAs of the shrink before a base launch (0: one per SM).
 int base_shrink_ctas(int T, int d_in, int d_out, int n_blk);
+// The shape launch_base would use on the current device; false when it is not prepared.
+bool base_launch_shape(int T, int d_in, int d_out, int n_blk, salt_base_shape *out);
 // A row-major bf16 tensor [rows][cols] as a 2-D TMA map, 128-byte swizzle (host).
 cudaError_t encode_map_2d(CUtensorMap *out, const uint16_t *base, int64_t cols, int64_t rows, uint32_t box_cols,
                           uint32_t box_rows);

@@ -1349,6 +1349,20 @@ salt_status salt_lora_apply_with_base(salt_ctx *ctx, const salt_segments *seg_, 
     return SALT_OK;
 }
 
+salt_status salt_base_get_shape(salt_ctx *ctx, const salt_segments *seg, int32_t layer, salt_base_shape *shape)
+{
+    if (!ctx || !seg || seg->ctx != ctx || !shape) return SALT_ERR_INVALID_ARG;
+    std::memset(shape, 0, sizeof *shape);
+    if (layer < 0 || layer >= ctx->n_layers)
+        return fail(ctx, SALT_ERR_LAYER_RANGE, "layer %d outside [0, %d)", layer, ctx->n_layers);
+    if (!seg->built) return fail(ctx, SALT_ERR_NOT_BUILT, "segments object was never built");
+    if (seg->T == 0) return SALT_OK;
+    if (!set_device(ctx)) return fail(ctx, SALT_ERR_CUDA, "cannot select device %d", ctx->device);
+    if (!base_launch_shape(seg->T, ctx->d_in[layer], ctx->d_out[layer], seg->n_blk_est, shape))
+        return fail(ctx, SALT_ERR_CUDA, "device %d is not prepared", ctx->device);
+    return SALT_OK;
+}
+
 salt_status salt_lora_apply(salt_ctx *ctx, const salt_segments *seg, int32_t layer, const void *x, void *y,
                             salt_stream_t stream)
 {

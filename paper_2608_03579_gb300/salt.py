@@ -67,6 +67,10 @@ class salt_ctx_info(ctypes.Structure):
                 ("block_users", ctypes.c_int32), ("reserved", ctypes.c_int32)]
 
 
+class salt_base_shape(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_int32) for k in ("cta_group", "tile_cols", "k_splits", "shrink_ctas", "units", "clusters")]
+
+
 _vp, _i32, _i64, _f32 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_float
 _SIGS = {
     "salt_abi_version": (_i32, []),
@@ -103,6 +107,7 @@ _SIGS = {
     "salt_host_pipe_wait": (ctypes.c_int, [_vp, _vp]),
     "salt_guard_check": (ctypes.c_int, [_vp, _vp, ctypes.POINTER(ctypes.c_int32)]),
     "salt_lora_apply_with_base": (ctypes.c_int, [_vp, _vp, _i32, _vp, _vp, _i32, _vp, _vp]),
+    "salt_base_get_shape": (ctypes.c_int, [_vp, _vp, _i32, ctypes.POINTER(salt_base_shape)]),
     "salt_fold_plan_create": (ctypes.c_int, [_vp, _i32, _i32, _vp, _vp, _i32, ctypes.POINTER(_vp)]),
     "salt_fold_plan_run": (ctypes.c_int, [_vp, _f32, _vp]),
     "salt_fold_plan_destroy": (None, [_vp]),
@@ -377,6 +382,13 @@ def salt_lora_apply(ctx, seg, layer: int, x, y, stream=None) -> None:
 def salt_lora_apply_with_base(ctx, seg, layer: int, x, W, layout: int, y, stream=None) -> None:
     """y = x W_base + the SALT delta (y written, not read)."""
     _check(_lib.salt_lora_apply_with_base(ctx, seg, layer, _ptr(x), _ptr(W), layout, _ptr(y), _stream(stream)), ctx)
+
+
+def salt_base_get_shape(ctx, seg, layer: int) -> dict:
+    """How salt_lora_apply_with_base would launch the layer's GEMM for the built batch."""
+    s = salt_base_shape()
+    _check(_lib.salt_base_get_shape(ctx, seg, layer, ctypes.byref(s)), ctx)
+    return {k: getattr(s, k) for (k, _) in salt_base_shape._fields_}
 
 
 def salt_lora_apply_static(ctx, seg, layer: int, x, y, stream=None) -> None:

@@ -100,17 +100,25 @@ def test_with_base_config3(salt_lib, oracle_mod, wl, layout):
                          f"with base, config 3 {w.layers[l][0]}, layout {layout}")
 
 
-@pytest.mark.parametrize("T,d_in,d_out", [
-    (1, 64, 64),          # one token, one K chunk, half a tile of columns
-    (24, 4096, 256),      # few tiles: K splits, one CTA a tile
-    (127, 136, 136), (128, 1032, 392),    # the last batches of one CTA a tile; remainders in K and N
-    (129, 1032, 392),     # the first batch of CTA pairs: one token in the second half
-    (257, 72, 264), (300, 4096, 128),     # a second M tile with an empty second half; K splits of pairs
-    (700, 520, 1288),     # more stages than the ring, several units a pair
+ONE, SEVERAL = "one unit a cluster", "several units a cluster"
+
+
+@pytest.mark.parametrize("T,d_in,d_out,cg,splits,units", [
+    (1, 64, 64, 1, False, ONE),           # one token, one K chunk, half a tile of columns
+    (24, 4096, 256, 1, True, ONE),        # few tiles: K splits that wait for each other
+    (24, 6144, 9728, 1, True, SEVERAL),   # K splits that leave their sums to the last
+    (100, 72, 20488, 1, False, SEVERAL),  # one CTA a tile, both accumulators, ring positions across units
+    (127, 136, 136, 1, False, ONE), (128, 1032, 392, 1, False, ONE),  # the last batches of one CTA a tile; remainders
+    (129, 1032, 392, 2, False, ONE),      # the first batch of CTA pairs: one token in the second half
+    (257, 72, 264, 2, False, ONE),        # a second M tile of one token
+    (300, 14336, 128, 2, True, ONE),      # K splits of pairs; a second M tile with an empty second half
+    (700, 520, 1288, 2, False, ONE),      # more stages than the ring
+    (2300, 136, 2056, 2, False, SEVERAL), # several units a pair, a last column tile of 8
 ])
 @pytest.mark.parametrize("layout", [0, 1])
-def test_with_base_tile_edges(salt_lib, oracle_mod, wl, layout, T, d_in, d_out):
-    """Every tile and split shape of the base kernel at its edges; users in
+def test_with_base_tile_edges(salt_lib, oracle_mod, wl, layout, T, d_in, d_out, cg, splits, units):
+    """Every tile and split shape of the base kernel at its edges (the launch
+    shape is checked, so a change of the plan cannot drop one); users in
     random order, stacks of one and of two 64-row chunks, tokens without a
     term; run twice (the split counters must be left at zero)."""
     from paper_2608_03579_gb300.runner import SaltRunner
@@ -126,13 +134,45 @@ def test_with_base_tile_edges(salt_lib, oracle_mod, wl, layout, T, d_in, d_out):
         r.pin_centroids()
         r.load_slots()
         r.build()
+        sh = salt_lib.salt_base_get_shape(r.ctx, r.seg, 0)
+        assert (sh["cta_group"], sh["k_splits"] > 1, sh["units"] > sh["clusters"]) == (cg, splits, units == SEVERAL), sh
         W = _weight(wl, 31, d_in, d_out, layout)
         got = _run(salt_lib, r, w, 0, W, layout)
         again = _run(salt_lib, r, w, 0, W, layout)
         assert r.device_error() == 0
         assert salt_lib.salt_guard_check(r.ctx, r.seg) == 0
     assert np.array_equal(got, again)
-    assert_close(got, _ref(oracle_mod, w, 0, W, layout), f"with base, {T} x {d_in} x {d_out}, layout {layout}")
+    rows = np.arange(T) if T < 2000 else np.unique(np.concatenate([np.arange(0, T, 7), [T - 1]]))
+    assert_close(got[rows], _ref(oracle_mod, w, 0, W, layout, rows=rows),
+                 f"with base, {T} x {d_in} x {d_out}, layout {layout}")
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+def test_with_base_consecutive_and_scattered_tiles(salt_lib, oracle_mod, wl, layout):
+    """Long user runs beside users in random order: pairs whose halves are both
+    consecutive tokens (x by tile loads), both gathered, and one of each."""
+    from paper_2608_03579_gb300.runner import SaltRunner
+    u = 2 + (wl.uniform(39, 1, 2240) * 28).astype(np.int32) % 28
+    for user, first, n in ((0, 0, 640), (1, 640, 70), (30, 1310, 500), (31, 1810, 128)):
+        u[first:first + n] = user
+    T, n_users, d_in, d_out = len(u), 32, 520, 776
+    w = wl.Workload("base_runs", 39, [("p", d_in, d_out)], 2, [64, 5], n_users, [1, 2] * (n_users // 2),
+                    dom_ids=(u >= 16).astype(np.int32), slot_ids=u)
+    w.y_mode = "zeros"
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        r.build()
+        perm = r.export()["perm"]
+        half = [bool((np.diff(perm[m:m + 128]) == 1).all()) for m in range(0, T - T % 256, 128)]
+        kinds = set(zip(half[::2], half[1::2]))
+        assert {(True, True), (False, False)} <= kinds and kinds & {(True, False), (False, True)}, kinds
+        assert salt_lib.salt_base_get_shape(r.ctx, r.seg, 0)["cta_group"] == 2
+        W = _weight(wl, 39, d_in, d_out, layout)
+        got = _run(salt_lib, r, w, 0, W, layout)
+        assert r.device_error() == 0
+        assert salt_lib.salt_guard_check(r.ctx, r.seg) == 0
+    assert_close(got, _ref(oracle_mod, w, 0, W, layout), f"with base, consecutive and scattered tiles, layout {layout}")
 
 
 @pytest.mark.parametrize("layout", [0, 1])
@@ -179,6 +219,7 @@ def test_with_base_splits_on_two_streams(salt_lib, oracle_mod, wl, T, d_in, d_ou
         try:
             for seg in segs:
                 salt.salt_build_segments(r.ctx, seg, w.dom_ids, w.slot_ids)
+                assert salt.salt_base_get_shape(r.ctx, seg, 0)["k_splits"] > 1
             x, Wd = bf16_tensor(w.x(0)), bf16_tensor(_weight(wl, 35, d_in, d_out, 1))
             ys = [torch.full((T, d_out), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(41)]
             salt.salt_lora_apply_with_base(r.ctx, r.seg, 0, x, Wd, 1, ys[0])
