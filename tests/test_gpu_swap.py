@@ -205,8 +205,7 @@ def test_batch_load_between_batches_on_side_stream(salt_lib, oracle_mod, wl):
 ])
 def test_batch_load_from_a_host_region(salt_lib, oracle_mod, wl, slots, shift):
     """Batches the swap kernel takes and ones it must not: ranks 1 and 2, blob
-    sizes that are no multiple of a CTA's piece, loaded twice so that a batch's
-    event is used again."""
+    sizes that are no multiple of a CTA's piece, each slot loaded twice."""
     from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
     salt = salt_lib
     T = 48
@@ -243,3 +242,136 @@ def test_batch_load_from_a_host_region(salt_lib, oracle_mod, wl, slots, shift):
         cents, res = oracle_tables(w, 1, version=lambda v: last.get(v, 0))
         ref = oracle_mod.apply(w.x(1), w.y_in(1), w.dom_ids, w.slot_ids, cents, res)
         assert_close(bf16_bits(y[turn]), ref, f"swap {turn} of {slots}")
+
+
+@pytest.mark.parametrize("layers,n_slots,kind", [
+    ([("p", 64, 64)], 300, "many"),                  # more blobs than a launch holds: two launches, one event
+    ([("p", 256, 264)] * 2, 6, "outside"),           # one blob in other pinned memory: copies
+    ([("p", 8192, 8192)] * 65, 4, "large"),          # blobs of 4.26 MB: copies
+    ([("p", 8192, 8192)] * 63, 4, "below large"),    # 4.13 MB: one launch
+])
+def test_batch_load_limits(salt_lib, oracle_mod, wl, layers, n_slots, kind):
+    """Batches at the limits of the swap kernel: every slot holds its blob."""
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
+    salt, l = salt_lib, len(layers) - 1
+    u = np.arange(2 * n_slots, dtype=np.int32) % n_slots
+    w = wl.Workload("swap_limits", 43, layers, 1, [1], n_slots, [2] * n_slots, dom_ids=np.zeros_like(u), slot_ids=u)
+    side, comp = torch.cuda.Stream(), torch.cuda.Stream()
+    with SaltRunner(w) as r:
+        assert (kind == "large") == (r.blob_bytes(2) > 4 << 20)
+        r.pin_centroids()
+        step = (r.blob_bytes(2) + 255) // 256 * 256
+        region = salt.salt_host_alloc(n_slots * step)
+        try:
+            blobs = [r.make_blob(v, out=None if kind == "outside" and v == 3 else
+                                 region.tensor[v * step:v * step + r.blob_bytes(2)]) for v in range(n_slots)]
+            salt.salt_residual_load_batch(r.ctx, list(range(n_slots)), blobs, side)
+            r.build(stream=comp)
+            x, y = bf16_tensor(w.x(l)), bf16_tensor(w.y_in(l))
+            salt.salt_lora_apply(r.ctx, r.seg, l, x, y, comp)
+            torch.cuda.synchronize()
+            assert r.device_error() == 0
+            assert salt.salt_guard_check(r.ctx, r.seg) == 0
+        finally:
+            torch.cuda.synchronize()
+            salt.salt_host_free(region)
+    cents, res = oracle_tables(w, l)
+    ref = oracle_mod.apply(w.x(l), w.y_in(l), w.dom_ids, w.slot_ids, cents, res)
+    assert_close(bf16_bits(y), ref, f"batch load, {kind}")
+
+
+def test_batch_events_are_used_again(salt_lib, oracle_mod, wl):
+    """Batches of which single loads and smaller batches replace a part: a
+    batch's event may be recorded again only once no slot's last load is that
+    batch.  Every batch is followed at once by a build and an apply that read
+    every slot; blobs large enough that a missed wait reads an old one."""
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
+    salt, n = salt_lib, 10
+    u = np.arange(40, dtype=np.int32) % n
+    w = wl.Workload("swap_events", 44, [("p", 256, 264)] + [("q", 8192, 8192)] * 12 + [("o", 264, 256)], 1, [1], n, [2] * n,
+                    dom_ids=np.zeros_like(u), slot_ids=u)
+    l = len(w.layers) - 1
+    # the event each is recorded in, and which others still hold a slot (event 0: the set-up's load of all ten)
+    turns = [[0, 1, 2, 3, 4, 5],   # 1; 0 keeps 6-9
+             [2],                  # the slot's own; 1 keeps 0 1 3 4 5
+             [6, 7, 8, 9],         # 2; then 0 is free
+             [0, 1, 3, 4],         # 0 again; 1 keeps 5
+             [5, 6, 7, 8, 9],      # 3; then 1 and 2 are free
+             [0, 1, 2, 3],         # 1 again; 0 keeps 4
+             [4, 5, 6, 7],         # 2 again; then 0 is free, 3 keeps 8 9
+             [8, 9, 0, 4],         # 0 again; then 3 is free
+             [1, 2, 3, 5, 6, 7]]   # 3 again
+    side, comp = torch.cuda.Stream(), torch.cuda.Stream()
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        step = (r.blob_bytes(2) + 255) // 256 * 256
+        region = salt.salt_host_alloc((n + sum(map(len, turns))) * step)
+        at = iter(range(0, region.nbytes, step))
+
+        def blob(slot, version):
+            a = next(at)
+            return r.make_blob(slot, version, out=region.tensor[a:a + r.blob_bytes(2)])
+
+        try:
+            salt.salt_residual_load_batch(r.ctx, list(range(n)), [blob(v, 0) for v in range(n)], side)
+            side.synchronize()
+            blobs = [[blob(v, t + 1) for v in slots] for t, slots in enumerate(turns)]
+            x = bf16_tensor(w.x(l))
+            ys = [bf16_tensor(w.y_in(l)) for _ in turns]
+            torch.cuda.synchronize()
+            for slots, bl, y in zip(turns, blobs, ys):
+                salt.salt_residual_load_batch(r.ctx, slots, bl, side)
+                r.build(stream=comp)
+                salt.salt_lora_apply(r.ctx, r.seg, l, x, y, comp)
+            torch.cuda.synchronize()
+            assert r.device_error() == 0
+            assert salt.salt_guard_check(r.ctx, r.seg) == 0
+        finally:
+            torch.cuda.synchronize()
+            salt.salt_host_free(region)
+    last = {v: 0 for v in range(n)}
+    for t, (slots, y) in enumerate(zip(turns, ys)):
+        last.update({v: t + 1 for v in slots})
+        cents, res = oracle_tables(w, l, version=lambda v: last[v])
+        ref = oracle_mod.apply(w.x(l), w.y_in(l), w.dom_ids, w.slot_ids, cents, res)
+        assert_close(bf16_bits(y), ref, f"after batch {t}")
+
+
+def test_batch_load_beside_base_calls(salt_lib, oracle_mod, wl):
+    """The swap kernel on a side stream while the base kernel runs (both fit an
+    SM): base results are those without it, and the slots hold their blobs."""
+    from paper_2608_03579_gb300.runner import SaltRunner, bf16_bits, bf16_tensor
+    salt, T, n = salt_lib, 256, 8
+    u = (wl.uniform(45, 1, T) * n).astype(np.int32) % n
+    w = wl.Workload("swap_base", 45, [("p", 1032, 2048)] + [("q", 8192, 8192)] * 20, 2, [16, 16], 2 * n, [2] * (2 * n),
+                    dom_ids=u % 2, slot_ids=u)
+    side, comp = torch.cuda.Stream(), torch.cuda.Stream()
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        step = (r.blob_bytes(2) + 255) // 256 * 256
+        region = salt.salt_host_alloc(n * step)
+        try:
+            blobs = [r.make_blob(n + i, 5, out=region.tensor[i * step:i * step + r.blob_bytes(2)]) for i in range(n)]
+            W = bf16_tensor(wl.normal_bf16(45, wl.stream_id(wl.K_AUX, 41), 1032 * 2048, 1032 ** -0.5).reshape(2048, 1032))
+            x, y0 = bf16_tensor(w.x(0)), bf16_tensor(w.y_in(0))
+            ys = [torch.empty(T, 2048, dtype=torch.bfloat16, device="cuda") for _ in range(24)]
+            r.build(stream=comp)
+            torch.cuda.synchronize()
+            for i, y in enumerate(ys):
+                if i == 2:
+                    salt.salt_residual_load_batch(r.ctx, list(range(n, 2 * n)), blobs, side)
+                salt.salt_lora_apply_with_base(r.ctx, r.seg, 0, x, W, 1, y, comp)
+            r.build(slot=w.slot_ids + n, stream=comp)
+            salt.salt_lora_apply(r.ctx, r.seg, 0, x, y0, comp)
+            torch.cuda.synchronize()
+            assert r.device_error() == 0
+            assert salt.salt_guard_check(r.ctx, r.seg) == 0
+        finally:
+            torch.cuda.synchronize()
+            salt.salt_host_free(region)
+    first = bf16_bits(ys[0])
+    assert all(np.array_equal(first, bf16_bits(y)) for y in ys[1:])
+    cents, res = oracle_tables(w, 0, version=lambda v: 5 if v >= n else 0)
+    ref = oracle_mod.apply(w.x(0), w.y_in(0), w.dom_ids, w.slot_ids + n, cents, res)
+    assert_close(bf16_bits(y0), ref, "slots loaded beside base calls")
