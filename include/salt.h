@@ -296,11 +296,10 @@ salt_status salt_residual_load(salt_ctx *ctx, int32_t slot, const void *host_blo
  * slot as it was).  On side_stream: one wait for the applies enqueued so
  * far on every segments object that refers to any of the slots, then the
  * blobs: by one kernel that reads them from host memory (four or more of at
- * most 4 MB, all in salt_host_alloc memory on 16-byte boundaries, the slots
- * distinct) and one
- * ready event, else by one cudaMemcpyAsync per blob, each followed by its
- * slot's ready event.  The result is that of n salt_residual_load calls in
- * order.  n == 0 does nothing.
+ * most 3 MiB, all in salt_host_alloc memory on 16-byte boundaries, the slots
+ * distinct) and one ready event, else by one cudaMemcpyAsync per blob, each
+ * followed by its slot's ready event.  The result is that of n
+ * salt_residual_load calls in order.  n == 0 does nothing.
  */
 salt_status salt_residual_load_batch(salt_ctx *ctx, int32_t n, const int32_t *slots, const void *const *host_blobs,
                                      salt_stream_t side_stream);

@@ -420,10 +420,12 @@ void slot_loaded(salt_ctx *ctx, int32_t slot, int32_t rank, int32_t batch)
 // Loads of one launch: at least this many blobs, in library host regions,
 // none larger than SWAP_LAUNCH_BYTES.  (A single blob is one copy-engine copy,
 // 6.5 us for 1.31 MB; between two copies the engine pays 2 us, which large
-// ones make up: a 32-layer 8B step with 64 blobs of 10.5 MB ran 3.32 ms by
-// copies and 3.70 by the launch, a four-layer one with 1.31 MB blobs 538 and 458 us.)
+// ones make up.)  8B decode steps of 1 to 32 layers, 512 tokens and 64 blobs,
+// by the launch and by copies, in us: blobs of 0.33 MB 150 / 233, 1.31 MB
+// 469 / 520, 1.97 MB 680 / 708, 2.62 MB 900 / 907, 3.28 MB 1123 / 1113, 3.93 MB
+// 1324 / 1297, 5.24 MB 1767 / 1695, 10.5 MB 3550 / 3255.
 constexpr int SWAP_LAUNCH_MIN = 4;
-constexpr uint64_t SWAP_LAUNCH_BYTES = 4 << 20;
+constexpr uint64_t SWAP_LAUNCH_BYTES = 3 << 20;
 
 // The loads of n checked blobs on `side`: readers first (every segments
 // object that names one of the slots waits for its uses, once), then the

@@ -247,8 +247,8 @@ def test_batch_load_from_a_host_region(salt_lib, oracle_mod, wl, slots, shift):
 @pytest.mark.parametrize("layers,n_slots,kind", [
     ([("p", 64, 64)], 300, "many"),                  # more blobs than a launch holds: two launches, one event
     ([("p", 256, 264)] * 2, 6, "outside"),           # one blob in other pinned memory: copies
-    ([("p", 8192, 8192)] * 65, 4, "large"),          # blobs of 4.26 MB: copies
-    ([("p", 8192, 8192)] * 63, 4, "below large"),    # 4.13 MB: one launch
+    ([("p", 8192, 8192)] * 48, 4, "large"),          # blobs of 3 MiB and a header: copies
+    ([("p", 8192, 8192)] * 47, 4, "below large"),    # the largest of such layers below: one launch
 ])
 def test_batch_load_limits(salt_lib, oracle_mod, wl, layers, n_slots, kind):
     """Batches at the limits of the swap kernel: every slot holds its blob."""
@@ -258,7 +258,7 @@ def test_batch_load_limits(salt_lib, oracle_mod, wl, layers, n_slots, kind):
     w = wl.Workload("swap_limits", 43, layers, 1, [1], n_slots, [2] * n_slots, dom_ids=np.zeros_like(u), slot_ids=u)
     side, comp = torch.cuda.Stream(), torch.cuda.Stream()
     with SaltRunner(w) as r:
-        assert (kind == "large") == (r.blob_bytes(2) > 4 << 20)
+        assert (kind == "large") == (r.blob_bytes(2) > 3 << 20)
         r.pin_centroids()
         step = (r.blob_bytes(2) + 255) // 256 * 256
         region = salt.salt_host_alloc(n_slots * step)
