@@ -103,6 +103,8 @@ struct FusedInfo {
 };
 constexpr size_t FUSED_SMEM = 1024 + RING_BYTES + (sizeof(FusedInfo) + 127) / 128 * 128;
 static_assert(FUSED_SMEM <= 227 * 1024, "shared memory exceeds the per-block limit");
+// (an SM has 228 KB, of which it keeps 1 KB a CTA: room for a swap CTA beside)
+static_assert(FUSED_SMEM + 2 * 1024 <= 228 * 1024, "shared memory exceeds what an SM has beside a swap CTA");
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
 {

@@ -5,12 +5,14 @@
 //
 // Bound by the host link.  A copy engine pays about 2 us between two copies
 // (64 blobs of 1.31 MB: 535 us one by one, 400 us as one copy); this kernel
-// takes 416 us.  Its CTAs (128 threads, at most 56 registers, no shared memory,
+// takes 416 us.  Its CTAs (128 threads, at most 48 registers, no shared memory,
 // the same shared-memory split) fit on an SM beside one CTA of the apply or
-// base kernels, so a swap on a side stream runs beside a step's applies.  An
-// 8B decode step of four layers with that swap: 538 us by copies, 458 with 20
-// CTAs, 545 with 12 (518 us alone), 481 with 28 and 588 with 64 (405 alone,
-// but they hold up the applies).
+// base kernels, so a swap on a side stream runs beside a step's applies: those
+// have 384 threads of 145 to 150 registers, handed out in eights, and 152 * 384
+// + 48 * 128 is within the SM's 65,536 (their shared memory is asserted where
+// they are).  An 8B decode step of four layers with that swap: 538 us by
+// copies, 458 with 20 CTAs, 545 with 12 (518 us alone), 481 with 28 and 588
+// with 64 (405 alone, but they hold up the applies).
 #include "salt_internal.cuh"
 
 #include <algorithm>
@@ -19,6 +21,9 @@ namespace salt {
 namespace {
 
 constexpr int SWAP_THREADS = 128;
+constexpr int SWAP_CTAS_PER_SM = 10;                        // caps the registers: 65,536 / 1,280 threads, in eights
+static_assert(65536 / (SWAP_CTAS_PER_SM * SWAP_THREADS) / 8 * 8 * SWAP_THREADS + 152 * APPLY_THREADS <= 65536,
+              "registers beside a CTA of the apply or base kernels");
 constexpr int SWAP_UNROLL = 8;                              // 16-byte loads a thread has in flight
 constexpr int SWAP_PIECE = SWAP_THREADS * SWAP_UNROLL;      // 16-byte units a CTA moves at a time
 constexpr int SWAP_CTAS = 20;                               // 0.33 MB in flight (above)
@@ -32,7 +37,7 @@ struct SwapParams {
     int32_t n;
 };
 
-__global__ void __launch_bounds__(SWAP_THREADS, 8) salt_swap_kernel(const __grid_constant__ SwapParams p)
+__global__ void __launch_bounds__(SWAP_THREADS, SWAP_CTAS_PER_SM) salt_swap_kernel(const __grid_constant__ SwapParams p)
 {
     int e = 0;
     for (uint32_t piece = blockIdx.x; piece < p.piece0[p.n]; piece += gridDim.x) {
