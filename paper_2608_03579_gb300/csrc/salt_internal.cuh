@@ -159,7 +159,6 @@ struct ApplyParams {
     const float *tok_sc;
     const int32_t *blk_res;
     int32_t rc_max;
-    int32_t min_nk;      // fewest 64-wide d_in chunks over the group's projections (caps the K splits)
     int32_t shared_x;    // every projection reads the same x (and d_in)
     int32_t tok_c4;      // 4-column pieces of a partial row that can hold anything (rc_max + r_max columns)
     uint32_t tok_c4_inv; // floor(2^32 / tok_c4) + 1: divides numbers below 2^12 by it (tok_c4 > 1)

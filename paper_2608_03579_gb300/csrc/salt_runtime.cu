@@ -1266,10 +1266,8 @@ salt_status apply_grouped(salt_ctx *ctx, const salt_segments *seg_, int32_t n, c
         units += (p.proj[i].d_out + 63) / 64;
     }
     p.n_unit_prefix[n] = units;
-    p.min_nk = 1 << 30;
     p.shared_x = 1;
     for (int i = 1; i < n; ++i) p.shared_x &= p.proj[i].x == p.proj[0].x && p.proj[i].d_in == p.proj[0].d_in;
-    for (int i = 0; i < n; ++i) p.min_nk = std::min(p.min_nk, (p.proj[i].d_in + 63) / 64);
     p.perm = seg->d.aperm;
     p.blk = seg->d.blk;
     p.counts = seg->d.counts;
@@ -1413,7 +1411,6 @@ salt_status salt_lora_apply_static(salt_ctx *ctx, const salt_segments *seg_, int
     p.n_proj = 1;
     p.n_unit_prefix[0] = 0;
     p.n_unit_prefix[1] = (pr.d_out + 63) / 64;
-    p.min_nk = (pr.d_in + 63) / 64;
     p.perm = seg->d.aperm;
     p.blk = seg->d.blk;
     p.counts = seg->d.counts;
