@@ -1207,9 +1207,16 @@ cudaError_t launch_apply(const ApplyParams &p, bool pdl, int ctas, int n_blk, cu
     cfg.numAttrs = pdl ? 1 : 0;
     // One kernel for all launches of a batch, whatever their projections: a
     // 3B MLP layer whose two launches took different ones ran 202 us, 190 with
-    // the same for both.
+    // the same for both.  The line lies where units can first be unsplit (eight
+    // projections a launch).  WHOLE / not, us a layer by its row blocks: 3B
+    // q/k/v 33.6 / 31.9 at 16, 40.5 / 38.2 at 24, 52.0 / 54.4 at 28, 72.3 / 75.0
+    // at 48, 104 / 120 at 100; 3B MLP 73 / 71 at 16, 118 / 116 at 32, 180 / 180 at
+    // 40, 290 / 320 at 100; 8B layer 154 / 148, 272 / 267, 404 / 406, 648 / 715 at
+    // the same.  So up to a third of the SMs in blocks WHOLE costs 2 to 6% where
+    // no launch has more than two projections, and gains 5 to 8% where one has
+    // three.
     return 8LL * n_blk > n_sm ? cudaLaunchKernelEx(&cfg, salt_apply_kernel<true>, p)
-                                                       : cudaLaunchKernelEx(&cfg, salt_apply_kernel<false>, p);
+                              : cudaLaunchKernelEx(&cfg, salt_apply_kernel<false>, p);
 }
 
 }  // namespace salt

@@ -40,8 +40,9 @@
 //
 // Measured against one CTA per 128 x 128 tile with cp.async for x, no K
 // split and the shrink run to its end first: a 3B MLP layer at 8192 tokens
-// 2937 -> 890 us (1.41 PFLOP/s), an 8B layer at 512 tokens 746 -> 324 us, at
-// 24 tokens 552 -> 175 us.  x by TMA tile::gather4 instead of the gather
+// 2939 -> 882 us (1.42 PFLOP/s), an 8B layer at 512 tokens 748 -> 322 us, at
+// 24 tokens 551 -> 175 us; single calls of 1 to 4096 tokens, 256 to 8192 wide,
+// 1.14 (4096 x 512 x 512) to 5.0 times as fast.  x by TMA tile::gather4 instead of the gather
 // warps took 3050 us for the first (about 90 cycles a four-row copy).
 #include <cuda_bf16.h>
 
@@ -228,7 +229,10 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     // block run side by side, so W is read from memory about once), split u % KS
     auto chunk_lo = [&](int s) { return nk * s / KS; };
     const bool in_out = p.w_layout == SALT_W_IN_OUT;
-    auto n_delta = [&](int mt, int s) { const int nd = (int)(info.mt_nd[mt >> 1] >> (16 * (mt & 1)) & 0xffffu); return nd > s ? (nd - s + KS - 1) / KS : 0; };
+    auto n_delta = [&](int mt, int s) {
+        const int nd = (int)(info.mt_nd[mt >> 1] >> (16 * (mt & 1)) & 0xffffu);
+        return nd > s ? (nd - s + KS - 1) / KS : 0;
+    };
 
     if (warp == 0) {
         // ============================================================ TMA
@@ -317,7 +321,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     wait_full(rp.slot, rp.phase, CG == 2);
                     tc_fence_after();
                     const uint64_t xd = x0 + rp.slot * st16, wd = wmn0 + rp.slot * st16;
-                            ok = __all_sync(0xffffffffu, ok);
+                    ok = __all_sync(0xffffffffu, ok);
                     const int steps = ok ? *reinterpret_cast<volatile uint8_t *>(&info.ksteps[rp.slot]) : 0;
                     if (elect_one()) {
                         for (int kk = 0; kk < steps; ++kk)
@@ -627,14 +631,21 @@ struct BasePlan {
     int cg, bn, ks, shrink_ctas;
 };
 
-// The launch's shape, by an estimate of its time in us (the constants are fits
-// to measured launches, 24 to 1024 tokens, d_in 4096 and 14336, d_out 1024 to
-// 14336): the tile width, the K splits, and the SMs the shrink gets.  Either
-// the shrink takes every SM and the K loop starts after it, or it takes
-// 24 or 48 beside the K loop on the others (only the delta waits for it):
-// worth it where the K loop is long or leaves SMs idle anyway, e.g. 24 tokens
-// of 4096 x 14336 45 -> 36 us beside, but 14336 x 4096 at 512 tokens 75 us in
-// turn against 89.
+// The launch's shape, by an estimate of its time in us: the tile width, the K
+// splits, and the SMs the shrink gets.  Either the shrink takes every SM and
+// the K loop starts after it, or it takes 24 or 48 beside the K loop on the
+// others (only the delta waits for it): worth it where the K loop is long or
+// leaves SMs idle anyway, e.g. 24 tokens of 4096 x 14336 45 -> 36 us beside,
+// but 14336 x 4096 at 512 tokens 75 us in turn against 89.
+// The constants are fits to measured launches of 24 to 1024 tokens, d_in 4096
+// and 14336, d_out 1024 to 14336; the estimate only ranks shapes, and its steps
+// (the tail at 8 tiles of tokens, no shrink beside above 2048 tokens) are rough.
+// Outside the fits, measured: 129, 200 and 300 tokens of 1024 x 1024 14.7, 14.9
+// and 15.2 us, of 4096 x 1024 24.4, 23.5 and 23.9; 2048 and 2049 tokens of
+// 4096 x 4096 62.9 and 62.9, of 8192 x 3072 86 and 113 (one wave more).  A shrink
+// beside above 2048 tokens gives as much as it takes: us in turn / beside at
+// 2560 tokens of 4096 x 1024 39.8 / 32.4, of 2048 x 2048 32.8 / 35.8, at 8192 of
+// 8192 x 3072 293 / 278, of 14336 x 512 150 / 158.
 BasePlan base_plan(int T, int d_in, int d_out, int n_blk, int n_sm, int max_pairs)
 {
     const int nk = (d_in + BK - 1) / BK, cg = T > BM ? 2 : 1;
@@ -657,7 +668,7 @@ BasePlan base_plan(int T, int d_in, int d_out, int n_blk, int n_sm, int max_pair
                 // (16 KB a chunk at 6 TB/s over the running CTAs, or by its
                 // own latency), a pair by its stages
                 const double active = (double)std::min<int64_t>(units, n_cl);
-                const double chunk = cg == 1 ? std::max(0.36, 0.41 * active / 152) : (bn == 256 ? 0.35 : 0.23);
+                const double chunk = cg == 1 ? std::max(0.36, 0.41 * active / n_sm) : (bn == 256 ? 0.35 : 0.23);
                 const double k_loop = ((nk + ks - 1) / ks) * chunk, tail = n_mt > 8 ? 1.0 : cg == 2 ? 9.0 : 4.0;
                 const bool share = units <= n_cl;
                 const double split = ks == 1 ? 0 : (m_rows / 128.0) * (bn / 128.0) * (share ? 2.0 : 0.5 + 0.8 * ks) + 2.0;

@@ -33,7 +33,7 @@
 // Bound by reading and writing W: two 8B layers (1.77 GB moved) go at 6.07
 // TB/s (a plain copy: 6.8).  One epilogue group that found each item's place
 // by 64-bit division and table reads was the bound before: two 8B layers in
-// a plan 363 -> 291 us, one 3072 x 3072 weight 10.1 -> 7.1 us.
+// a plan 363 -> 291 us, one 3072 x 3072 weight 10.1 -> 8.2 us.
 #include "salt_async.cuh"
 #include "salt_internal.cuh"
 #include "salt_pipe.cuh"

@@ -79,7 +79,7 @@ struct salt_segments {
     bool device_ids = false;
     int T = 0;
     int n_blk_bound = 0;                       // launch bound on the row blocks of the last build
-    int n_blk_est = 1;                         // about how many there are (shapes launches only)
+    int n_blk_est = 1;                         // about how many there are (shapes launches only; a guess for device ids)
     ApplyWork work{};                          // V tiles of the apply path
     std::vector<uint8_t> refs;                 // slots named by the last build (host ids)
     cudaStream_t build_stream = nullptr;
@@ -1160,6 +1160,9 @@ salt_status salt_build_segments_gamma(salt_ctx *ctx, salt_segments *seg, const i
     seg->T = T;
     if (dev_ids) std::fill(seg->refs.begin(), seg->refs.end(), 1);
     else seg->refs.swap(refs);
+    // (device ids: half the bound, which no data backs; it shapes the base
+    // launch only: 512 tokens of 4096 x 4096 in 64 users 29.8 us against 24.4 with
+    // host ids, 1024 x 1024 and 2048 tokens and more the same)
     seg->n_blk_est = std::max(1, std::min(block_bound_loose(ctx, T), seg->work.blk_cap) / 2);
     if (T == 0) seg->n_blk_bound = 0;
     else if (dev_ids) seg->n_blk_bound = std::min(block_bound_loose(ctx, T), seg->work.blk_cap);
