@@ -414,8 +414,8 @@ salt_status salt_lora_apply_grouped(salt_ctx *ctx, const salt_segments *seg, int
  * y are 16-byte aligned, y does not overlap x or W.  Two launches on
  * `stream`: the apply kernel writing the row blocks' V tiles into the
  * segments workspace, then one tcgen05 kernel that runs the GEMM over
- * 128-token tiles in grouped order and adds each overlapping row block's
- * V * [B_c; b_u] into the same accumulator.  Asynchronous; the workspace
+ * tiles of 128 or 256 tokens in grouped order and adds each overlapping row
+ * block's V * [B_c; b_u] into the same accumulator.  Asynchronous; the workspace
  * is shared with salt_lora_apply on the same segments object (stream
  * order keeps them apart).  A captured call may be replayed after the
  * segments object was rebuilt with at most as many tokens as it had at the
