@@ -10,8 +10,9 @@
 // kernel runs the GEMM over tiles of tokens in grouped order and, for every
 // row block overlapping a tile, adds V_ext * Stack_B into the same
 // tensor-memory accumulator: further K chunks whose A operand holds the
-// block's V rows at their tile rows and zeros elsewhere.  Tokens with no term
-// are in no block and get x W_base alone.
+// block's V rows at their tile rows and zeros elsewhere, and whose MMAs leave
+// the other rows' lanes alone.  Tokens with no term are in no block and get
+// x W_base alone.
 //
 // CG = 2 (batches of more than 128 tokens): a cluster of two CTAs computes a
 // 256-token x BN tile with cta_group::2 MMAs.  Each CTA loads its own 128
@@ -75,17 +76,18 @@ struct BaseInfo {
     uint64_t accf[2], acce[2];
     int32_t mt_b0[MT_MAX], mt_b1[MT_MAX];  // row blocks overlapping M tile: [b0, b1)
     uint32_t mt_nd[MT_MAX / 2];            // its delta chunks (at most 512), two tiles to a word
-    int16_t mt_x0[MT_MAX];                 // its first token where this CTA's rows are consecutive tokens, else -1
-    uint32_t mt_peer[MT_MAX / 32];         // bit: the pair's second CTA gathers the tile's rows
-    uint8_t ksteps[NST_MAX];               // a delta stage's K = 16 steps
-    alignas(16) uint32_t token[4];         // copied by the second CTA's gather warps to signal the first
+    uint16_t mt_x0[MT_MAX];                // its first token, X_GATHER and X_PEER
     uint32_t tmem;
     uint32_t shares;
+    uint32_t dstage[NST_MAX];              // a delta stage: its K = 16 steps, first and end row of its block in the tile (10 bits each)
+    alignas(16) uint32_t token[4];         // copied by the second CTA's gather warps to signal the first
 };
 constexpr size_t BASE_SMEM = 1024 + BASE_RING + (sizeof(BaseInfo) + 15) / 16 * 16;
 // (an SM has 228 KB, of which it keeps 1 KB a CTA: room for a swap CTA beside)
 static_assert(BASE_SMEM + 2 * 1024 <= 228 * 1024, "shared memory exceeds what an SM has beside a swap CTA");
-static_assert(SALT_MAX_TOKENS <= 32767, "mt_x0 holds a token index");
+constexpr uint16_t X_GATHER = 1u << 15;  // this CTA's rows of the tile are not consecutive tokens
+constexpr uint16_t X_PEER = 1u << 14;    // the pair's second CTA's are not
+static_assert(SALT_MAX_TOKENS <= X_PEER, "mt_x0 holds a token index below the flags");
 // A gather warp fills every GWN-th stage and waits only for its own slots'
 // phases; with at least GWN stages a slot's barrier is never two phases
 // behind the one it waits for (a parity wait could not tell).
@@ -178,7 +180,6 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         info.mt_b0[i] = 0x7fffffff;
         info.mt_b1[i] = 0;
         info.mt_nd[i >> 1] = 0;
-        info.mt_peer[i >> 5] = 0;
     }
     __syncthreads();
     // Row blocks lie in grouped order and hold at most TM tokens, so each
@@ -199,18 +200,17 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
     // Tiles whose rows are consecutive tokens (runs of a prefill batch) take x
     // by plain TMA tiles; a batch of one tile is not looked at.
     for (int t = warp; t < n_mt; t += BASE_THREADS / 32) {
+        uint32_t x = 0;
         for (int h = rank; h < CG; ++h) {  // the first CTA looks at both halves
             const int m0 = (t * CG + h) * BM, rows = min(BM, T - m0);
-            int x0 = -1;
-            if (CG == 2 && rows > 0) {
-                x0 = p.perm[m0];
-                bool lin = true;
-                for (int i = lane; i < rows; i += 32) lin = lin && p.perm[m0 + i] == x0 + i;
-                if (!__all_sync(0xffffffffu, lin)) x0 = -1;
-            }
-            if (lane == 0 && h == rank) info.mt_x0[t] = (int16_t)x0;
-            if (lane == 0 && h == 1 && x0 < 0) atomicOr(&info.mt_peer[t >> 5], 1u << (t & 31));
+            bool lin = CG == 2 && rows > 0;
+            const int x0 = lin ? p.perm[m0] : 0;
+            for (int i = lane; i < rows && lin; i += 32) lin = p.perm[m0 + i] == x0 + i;
+            lin = __all_sync(0xffffffffu, lin);
+            if (h == rank) x |= lin ? (uint32_t)x0 : X_GATHER;
+            if (h == 1 && !lin) x |= X_PEER;
         }
+        if (lane == 0) info.mt_x0[t] = (uint16_t)x;
     }
     tc_fence_before();
     cta_or_cluster_sync<CG>();
@@ -248,8 +248,8 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         };
         for (int u = cl; u < n_units && ok; u += n_cl) {
             const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
-            const int k1 = chunk_lo(s + 1), x0 = info.mt_x0[mt];
-            const bool peer = CG == 2 && rank == 0 && (info.mt_peer[mt >> 5] >> (mt & 31) & 1u);
+            const int k1 = chunk_lo(s + 1), xt = info.mt_x0[mt], x0 = xt & (X_PEER - 1);
+            const bool lin = !(xt & X_GATHER), peer = CG == 2 && rank == 0 && (xt & X_PEER);
             for (int kc = chunk_lo(s); kc < k1 && ok; ++kc, advance()) {
                 next_slot();
                 if (!ok) break;
@@ -257,8 +257,8 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     const uint32_t ws = ring32 + rp.slot * stage + x_bytes;
                     const uint32_t fb = leader_addr<CG>(bar(info.full[rp.slot]));
                     const int k0 = kc * BK;
-                    mbar_expect_tx_cluster<CG>(fb, (uint32_t)NB * 128u + (x0 >= 0 ? x_bytes : 0u) + (peer ? BULK_SIGNAL_BYTES : 0u));
-                    if (x0 >= 0) tma_load_2d_cg<CG>(ws - x_bytes, &p.xmap, k0, x0, fb);
+                    mbar_expect_tx_cluster<CG>(fb, (uint32_t)NB * 128u + (lin ? x_bytes : 0u) + (peer ? BULK_SIGNAL_BYTES : 0u));
+                    if (lin) tma_load_2d_cg<CG>(ws - x_bytes, &p.xmap, k0, x0, fb);
                     if (in_out) {
                         // W[d_in][d_out]: boxes of 64 K rows x 64 N columns (MN-major)
                         for (int h = 0; h < NB / 64; ++h) tma_load_2d_cg<CG>(ws + h * 8192, &p.wmap, n0 + 64 * h, k0, fb);
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                 if (lt >= 2) wait_bar(info.acce[buf], ((lt - 2) >> 1) & 1);
                 tc_fence_after();
                 uint32_t accum = 0;
-                const bool peer = CG == 2 && (info.mt_peer[mt >> 5] >> (mt & 31) & 1u);
+                const bool peer = CG == 2 && (info.mt_x0[mt] & X_PEER);
                 for (int n = chunk_lo(s + 1) - chunk_lo(s); n > 0; --n, rp.advance(1, nst)) {
                     wait_full(rp.slot, rp.phase, peer);
                     tc_fence_after();
@@ -317,19 +317,24 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                     __syncwarp();
                     accum = 1;
                 }
+                // (added to at least one K chunk's product: KS <= nk)
                 for (int n = n_delta(mt, s); n > 0; --n, rp.advance(1, nst)) {
                     wait_full(rp.slot, rp.phase, CG == 2);
                     tc_fence_after();
                     const uint64_t xd = x0 + rp.slot * st16, wd = wmn0 + rp.slot * st16;
                     ok = __all_sync(0xffffffffu, ok);
-                    const int steps = ok ? *reinterpret_cast<volatile uint8_t *>(&info.ksteps[rp.slot]) : 0;
+                    // only the block's own rows: an infinity in its B times the
+                    // other rows' zeros would be a NaN in theirs
+                    const uint32_t ds = ok ? *reinterpret_cast<volatile uint32_t *>(&info.dstage[rp.slot]) : 0u;
+                    const int steps = (int)(ds & 0x3ffu);
+                    uint32_t off[4 * CG];
+                    lanes_off<CG>((int)(ds >> 10 & 0x3ffu), (int)(ds >> 20), off);
                     if (elect_one()) {
                         for (int kk = 0; kk < steps; ++kk)
-                            umma_bf16_cg<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, kk > 0 ? 1u : accum);
+                            umma_bf16_cg_lanes<CG>(acc, xd + kk * 2, wd + kk * 128, id_mn, off);
                         umma_commit_cg<CG>(bar(info.empty[rp.slot]));
                     }
                     __syncwarp();
-                    accum = 1;
                 }
                 if (elect_one()) umma_commit_cg<CG>(bar(info.accf[buf]));
                 __syncwarp();
@@ -373,7 +378,7 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
         for (int u = cl; u < n_units && ok; u += n_cl) {
             const int tile = u / KS, s = u - tile * KS, mt = tile % n_mt, n0 = tile / n_mt * BN + rank * NB;
             const int m0 = (mt * CG + rank) * BM;
-            const bool lin = info.mt_x0[mt] >= 0;
+            const bool lin = !(info.mt_x0[mt] & X_GATHER);
             if (mt != mt_of && !lin) {
                 mt_of = mt;
                 rows = max(0, min(BM, T - m0));
@@ -465,7 +470,11 @@ __global__ void __launch_bounds__(BASE_THREADS, 1) salt_base_kernel(const __grid
                             const bool in = sp != nullptr && col < p.d_out;
                             cp_async16(ws + (c >> 3) * 8192 + swz128(k, c & 7), in ? sp + col : p.x, in);
                         }
-                        if (lane == 0) info.ksteps[rp.slot] = (uint8_t)(kn >> 4);
+                        if (lane == 0) {
+                            const int r0 = start - mt * (BM * CG);  // the block's first row in the tile
+                            info.dstage[rp.slot] = (uint32_t)(kn >> 4) | (uint32_t)max(r0, 0) << 10 |
+                                                   (uint32_t)min(r0 + M, BM * CG) << 20;
+                        }
                         finish();
                         mine -= 1;  // this stage itself
                     }

@@ -259,6 +259,38 @@ __device__ __forceinline__ void umma_bf16_cg(uint32_t d_tmem, uint64_t adesc, ui
             "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
     }
 }
+// The lanes of D that an MMA updating only its rows [lo, hi) must not write
+// (rows past 127 are the second CTA's lanes): a bit each, a word per lane of
+// the warp and then everyone's copy.  Whole warp.
+template <int CG>
+__device__ __forceinline__ void lanes_off(int lo, int hi, uint32_t (&off)[4 * CG])
+{
+    const int at = 32 * (int)(threadIdx.x & (4 * CG - 1));
+    const int a = min(max(lo - at, 0), 32), b = min(max(hi - at, 0), 32);
+    uint32_t on;
+    asm("bmsk.clamp.b32 %0, %1, %2;\n" : "=r"(on) : "r"(a), "r"(max(b - a, 0)));
+#pragma unroll
+    for (int j = 0; j < 4 * CG; ++j) off[j] = ~__shfl_sync(0xffffffffu, on, j);
+}
+// D += A * B^T for one K=16 step in the other lanes; those keep their values,
+// whatever B holds.
+template <int CG>
+__device__ __forceinline__ void umma_bf16_cg_lanes(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                   const uint32_t (&off)[4 * CG])
+{
+    if constexpr (CG == 1) {
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, 1, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%4, %5, %6, %7}, "
+            "p;\n}\n" ::"r"(d_tmem),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(off[0]), "r"(off[1]), "r"(off[2]), "r"(off[3]));
+    } else {
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, 1, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, {%4, %5, %6, %7, "
+            "%8, %9, %10, %11}, p;\n}\n" ::"r"(d_tmem),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(off[0]), "r"(off[1]), "r"(off[2]), "r"(off[3]), "r"(off[4]), "r"(off[5]),
+            "r"(off[6]), "r"(off[7]));
+    }
+}
 // arrive on the barrier at this address of every CTA of the pair once the
 // issuing thread's tcgen05 operations so far have completed
 template <int CG>

@@ -283,3 +283,33 @@ def test_with_base_replayed_after_rebuilds(salt_lib, oracle_mod, wl, T, later):
             if done:
                 ref = oracle_mod.apply(w.x(0)[:n], None, dom, slot, cents, res, w_base=W, w_layout=1)
                 assert_close(got[:n], ref, f"captured on {T} tokens, replayed on {n}")
+
+
+@pytest.mark.parametrize("T,d_out", [(100, 264), (128, 2048), (400, 264), (512, 1032)])
+def test_with_base_infinity_stays_in_its_block(salt_lib, oracle_mod, wl, T, d_out):
+    """A user whose residual holds infinities: tokens outside the row blocks
+    that the user's tokens are in get the values they would without that user."""
+    from paper_2608_03579_gb300.runner import SaltRunner
+    n_users, d_in, bad = 40, 264, 21
+    u = (wl.uniform(47, 1, T) * n_users).astype(np.int32) % n_users
+    w = wl.Workload("base_inf", 47, [("p", d_in, d_out)], 4, [64, 5, 16, 64], n_users, [2] * n_users,
+                    dom_ids=(u % 4).astype(np.int32), slot_ids=u)
+    w.y_mode = "zeros"
+    with SaltRunner(w) as r:
+        r.pin_centroids()
+        r.load_slots()
+        blob = r.make_blob(bad)
+        blob[256 + 2 * 2 * d_in:].view(torch.int16).fill_(0x7F80)  # both rows of B
+        salt_lib.salt_residual_load(r.ctx, bad, blob)
+        r.build()
+        exp = r.export()
+        beside = np.zeros(T, bool)
+        for start, n, _ in exp["blocks"]:
+            tokens = exp["perm"][start:start + n]
+            beside[tokens] |= (u[tokens] == bad).any()
+        W = _weight(wl, 47, d_in, d_out, 1)
+        got = _run(salt_lib, r, w, 0, W, 1)
+        assert r.device_error() == 0
+    rows = np.flatnonzero(~beside)
+    assert 0 < len(rows) < T
+    assert_close(got[rows], _ref(oracle_mod, w, 0, W, 1, rows=rows), f"beside an infinity, {T} tokens")
