@@ -8,7 +8,7 @@
 // takes 416 us.  Its CTAs (128 threads, at most 48 registers, no shared memory,
 // the same shared-memory split) fit on an SM beside one CTA of the apply or
 // base kernels, so a swap on a side stream runs beside a step's applies: those
-// have 384 threads of 145 to 150 registers, handed out in eights, and 152 * 384
+// have 384 threads of 145 to 151 registers, handed out in eights, and 152 * 384
 // + 48 * 128 is within the SM's 65,536 (their shared memory is asserted where
 // they are).  An 8B decode step of four layers with that swap: 538 us by
 // copies, 458 with 20 CTAs, 545 with 12 (518 us alone), 481 with 28 and 588
